@@ -402,12 +402,15 @@ int mw3_product_probabilities(mw3_ctx* ctx, double* P);
  *                "prod_points" (read only) is the number of distinct stencil columns
  *   "f64_tc"     0/1: MW3_FP64 angular step on the tensor cores as exact products of 8-bit
  *                digits (ngamma <= 192; default 1), or FP64 GEMMs on the CUDA cores
- *   "tc_wait_limit" 0..2^22: polls of each bounded mbarrier wait of the tile-major angular
- *                step (default 2^22). A wait that runs out makes its CTA stop, wait (with the
- *                full 2^22 bound) for the tensor-core work already committed, free its tensor
- *                memory and set the error word that mw3_propagate returns as
- *                MW3_ERR_TIMEOUT; 0 makes every wait run out (the failure-detection test).
- *                The context is not usable for propagation after a timeout; the device is.
+ *   "tc_wait_limit" 0..2^22: polls of each bounded mbarrier wait of the tensor-core angular
+ *                steps and the tensor-core flush (default 2^22). A wait that runs out makes its
+ *                CTA stop, wait (with the full 2^22 bound) for the tensor-core work already
+ *                committed, free its tensor memory and set an error word. mw3_propagate (and a
+ *                probability read or checkpoint that flushes pending iterations) returns it
+ *                as MW3_ERR_TIMEOUT, after which the context is not usable for propagation;
+ *                mw3_apply_hs, mw3_lanczos and the bound-state calls return it and leave the
+ *                propagation state alone. 0 makes every wait run out (the failure-detection
+ *                tests).
  * Values outside a key's range return MW3_ERR_BAD_ARG. mw3_get_tuning reads a key. */
 int mw3_set_tuning(mw3_ctx* ctx, const char* key, long value);
 long mw3_get_tuning(const mw3_ctx* ctx, const char* key);

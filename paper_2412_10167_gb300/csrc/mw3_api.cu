@@ -82,6 +82,7 @@ struct mw3_ctx {
   // host-to-device state uploads: a copy stream and one event per block group, so that a
   // group's conversion and gamma transform overlap the next group's copy
   cudaStream_t up_stream = nullptr;
+  int* tc_word = nullptr;        // page-locked copy of the error words (see tc_fetch)
   bool up_direct_last = false;   // the last state upload read mapped host memory directly
   cudaEvent_t up_ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
   bool own_stream = false;
@@ -515,6 +516,23 @@ int transform_download(mw3_ctx* ctx, const char* src_name, double* dst) {
   return MW3_OK;
 }
 
+// Did a bounded wait of the tensor-core kernels queued so far run out? Word 0 of "tc_err" belongs
+// to the propagation (iterations and flushes; it stays set, the state and the sums are damaged),
+// word 1 to H_s applications, whose results alone are lost: it is cleared for the next one.
+// tc_fetch queues the read (into page-locked memory: no wait of its own), tc_result looks at it
+// after the caller's synchronisation.
+int tc_fetch(mw3_ctx* ctx, int word) {
+  if (!dptr(ctx, "tc_err")) return MW3_OK;
+  CK(cudaMemcpyAsync(ctx->tc_word + word, (int*)dptr(ctx, "tc_err") + word, sizeof(int),
+                     cudaMemcpyDeviceToHost, ctx->stream));
+  return MW3_OK;
+}
+int tc_result(mw3_ctx* ctx, int word) {
+  if (!dptr(ctx, "tc_err") || !ctx->tc_word[word]) return MW3_OK;
+  if (word) CK(cudaMemsetAsync((int*)dptr(ctx, "tc_err") + word, 0, sizeof(int), ctx->stream));
+  return ctx->fail(MW3_ERR_TIMEOUT, "tensor-core step: an mbarrier wait timed out");
+}
+
 const char* state_name(const mw3_ctx* ctx, bool current) {
   return (current == (ctx->cur == 0)) ? "q0" : "q1";
 }
@@ -668,6 +686,7 @@ void mw3_destroy(mw3_ctx* ctx) {
     for (auto e : ctx->up_ev)
       if (e) cudaEventDestroy(e);
     if (ctx->up_stream) cudaStreamDestroy(ctx->up_stream);
+    if (ctx->tc_word) cudaFreeHost(ctx->tc_word);
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
   }
   delete ctx;
@@ -1030,6 +1049,8 @@ static int finish_potential(mw3_ctx* ctx, double vcut, double tcut, double erot)
   }
   ctx->kh64 = ctx->precision == MW3_FP64 ? angular_f64_kh(ng) : 0;
   if (ctx->kh64 > 0 && (st = upload_f64_tables(ctx))) return st;
+  if (dptr(ctx, "tc_err") && !ctx->tc_word)
+    CK(cudaHostAlloc((void**)&ctx->tc_word, 2 * sizeof(int), cudaHostAllocDefault));
   if ((st = upload_real(ctx, "coef", ctx->coef))) return st;
   if ((st = upload_real(ctx, "fR", ctx->fR))) return st;
   if ((st = upload_real(ctx, "fr", ctx->fr))) return st;
@@ -1946,7 +1967,8 @@ int step(mw3_ctx* ctx, int slot, bool first, bool timed, int mode = 0, real* hs_
     a.dj = B.dj;
     a.out = (double*)hs_out;
     a.npart = mode == 0 ? (double*)dptr(ctx, "npart") : nullptr;
-    a.err = (int*)dptr(ctx, "tc_err");
+    a.err = (int*)dptr(ctx, "tc_err") + mode;
+    a.wait_limit = ctx->tune.tc_wait_limit;
     a.alpha = first ? 1.0 : 2.0;
     a.beta = first ? 0.0 : 1.0;
     a.ncol = ctx->ncol;
@@ -1983,7 +2005,7 @@ int step(mw3_ctx* ctx, int slot, bool first, bool timed, int mode = 0, real* hs_
     a.dj = B.dj;
     a.out = (float*)hs_out;
     a.npart = mode == 0 ? (double*)dptr(ctx, "npart") : nullptr;
-    a.err = (int*)dptr(ctx, "tc_err");
+    a.err = (int*)dptr(ctx, "tc_err") + mode;
     a.wait_limit = ctx->tune.tc_wait_limit;
     a.erot = (float)ctx->erot;
     a.alpha = first ? 1.0f : 2.0f;
@@ -2089,7 +2111,7 @@ int flush(mw3_ctx* ctx, int nvalid, bool timed) {
   if (std::is_same<real, float>::value && ctx->tc_ok && ctx->tune.flush_tc) {
     LK(launch_flush_tc((const float*)B.ph, (const float*)B.cut, ctx->NC, ctx->tune.kb, nvalid, ctx->nJ,
                        ctx->an.nE, B.colbase, B.ncols, B.accoff, ctx->max_cols, B.acc,
-                       (int*)dptr(ctx, "tc_err"), st));
+                       ctx->tune.tc_wait_limit, (int*)dptr(ctx, "tc_err"), st));
   } else {
     LK(launch_sums_flush<real>(B.ph, B.cut, ctx->NC, ctx->tune.kb, nvalid, ctx->nJ, ctx->an.nE,
                                B.colbase, B.ncols, B.accoff, ctx->max_cols, B.acc, st));
@@ -2128,12 +2150,11 @@ int check_norms(mw3_ctx* ctx, int slot0, int n) {
     CK(cudaMemcpyAsync(ac.data(), (const double*)dptr(ctx, "acbuf") + (size_t)slot0 * ctx->nJ,
                        ac.size() * 8, cudaMemcpyDeviceToHost, ctx->stream));
   }
-  int tc_err = 0;
-  if (dptr(ctx, "tc_err"))
-    CK(cudaMemcpyAsync(&tc_err, dptr(ctx, "tc_err"), 4, cudaMemcpyDeviceToHost, ctx->stream));
+  int st = tc_fetch(ctx, 0);
+  if (st) return st;
   CK(cudaStreamSynchronize(ctx->stream));
   collect_times(ctx);
-  if (tc_err) return ctx->fail(MW3_ERR_TIMEOUT, "tensor-core step: an mbarrier wait timed out");
+  if ((st = tc_result(ctx, 0))) return st;
   ctx->norm_trace.insert(ctx->norm_trace.end(), h.begin(), h.end());
   ctx->ac_trace.insert(ctx->ac_trace.end(), ac.begin(), ac.end());
   for (double v : h)
@@ -2195,11 +2216,11 @@ int propagate_impl(mw3_ctx* ctx, long nsteps) {
 int flush_pending(mw3_ctx* ctx) {
   if (ctx->ring_n == 0 || ctx->host_only) return MW3_OK;
   const int n = ctx->ring_n;
-  const int st = ctx->precision == MW3_FP64 ? flush<double>(ctx, n, false) : flush<float>(ctx, n, false);
-  if (st) return st;
+  int st = ctx->precision == MW3_FP64 ? flush<double>(ctx, n, false) : flush<float>(ctx, n, false);
+  if (st || (st = tc_fetch(ctx, 0))) return st;
   ctx->ring_n = 0;
   CK(cudaStreamSynchronize(ctx->stream));
-  return MW3_OK;
+  return tc_result(ctx, 0);
 }
 
 void incoming_a2(mw3_ctx* ctx, std::vector<double>& a2);
@@ -2341,8 +2362,9 @@ int lanczos_run(mw3_ctx* ctx, int m, bool accumulate) {
     w = t;
   }
   ctx->buf[qname].p = saved;
+  const int fst = tc_fetch(ctx, 1);
   CK(cudaStreamSynchronize(st));
-  return status;
+  return status ? status : (fst ? fst : tc_result(ctx, 1));
 }
 
 // Lanczos coefficients of m steps from the host start vector v0 (grid values), per J.
@@ -2666,8 +2688,8 @@ int mw3_apply_hs(mw3_ctx* ctx, const double* q, double* out) {
     st = step<float>(ctx, 0, true, false, 1, (float*)dptr(ctx, "hs_out"));
   ctx->buf[qname].p = saved;
   ctx->cur = cur0;
-  if (st) return st;
-  return transform_download(ctx, "hs_out", out);
+  if (st || (st = tc_fetch(ctx, 1)) || (st = transform_download(ctx, "hs_out", out))) return st;
+  return tc_result(ctx, 1);
 }
 
 long mw3_norm_trace(mw3_ctx* ctx, double* out, long n) {

@@ -81,8 +81,8 @@ struct Tuning {
                     // default: 0.380 against 0.399 ms per step on config 2)
   int prod_gather;  // product-channel node sums: stencil columns gathered plane-major first
                     // (1) or read as 4 x 4 stencils straight from the state (0)
-  long tc_wait_limit;   // polls of the tile-major angular step's bounded waits (2^22; smaller
-                        // values serve the failure-detection test)
+  long tc_wait_limit;   // polls of the tensor-core kernels' bounded waits (2^22; smaller values
+                        // serve the failure-detection tests)
   int f64_tc;       // MW3_FP64: the angular step as exact digit products on the tensor cores
                     // (mw3_f64tc.cu; 1, the default where it applies) or CUDA-core GEMMs (0)
 };
@@ -311,8 +311,8 @@ struct TcArgs {
   float* out;           // mode 1: H_s c
   double* npart;        // [group][tile] sums of squares of c_(k+1)
   int* err;             // set on a wait that timed out
-  long wait_limit;      // polls of a bounded wait in the tile-major form (the wait for the MMAs
-                        // of an expired phase before tensor memory is freed keeps 2^22)
+  long wait_limit;      // polls of a bounded wait (the wait for the MMAs of an expired phase
+                        // before tensor memory is freed keeps 2^22)
   float erot, alpha, beta;
   long ncol, npts;
   int ng, kp, NR, nelec, mode, ntiles, tmem_cols;
@@ -360,7 +360,8 @@ struct F64Args {
   const DevJ* dj;
   double* out;                // mode 1: H_s c
   double* npart;              // [group][tile] sums of squares of c_(k+1)
-  int* err;
+  int* err;                   // set on a wait that timed out
+  long wait_limit;            // polls of a bounded wait (as in TcArgs)
   double alpha, beta;
   long ncol, npts;
   int ng, kh, NR, nr, nelec, mode, ntiles, ngroups, nsm;
@@ -370,7 +371,8 @@ cudaError_t launch_angular_f64(const F64Args& a, const int* g_begin, int nJ, dou
 // Energy-sum flush on the tensor cores (FP32 ring, split-TF32, FP64 accumulators).
 cudaError_t launch_flush_tc(const float* ph, const float* cut, long ncut_total, int kb, int nvalid, int nJ,
                             int nE, const long* colbase, const long* ncols, const long* accoff,
-                            long max_cols, double* acc, int* err, cudaStream_t st);
+                            long max_cols, double* acc, long wait_limit, int* err,
+                            cudaStream_t st);
 int angular_tc3_kh(int ng, int nelec);   // 0 when the parity-split form does not apply
 int angular_tc4_kh(int ng, int nelec);   // 0 when the streamed parity-split form does not apply
 size_t angular_tc_smem(int kp);

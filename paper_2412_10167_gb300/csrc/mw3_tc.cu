@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc(TcArgs a) {
       issue_split_gemm(tmem + (uint32_t)(L * kp), Ahi, Alo, Bhi, Blo, kp, idesc);
       mma_commit(mb);
     }
-    ok = __syncthreads_and(mbar_wait(mb, phase) ? 1 : 0) != 0;  // CTA-uniform
+    ok = __syncthreads_and(mbar_wait(mb, phase, a.wait_limit) ? 1 : 0) != 0;  // CTA-uniform
     phase ^= 1;
     asm volatile("tcgen05.fence::after_thread_sync;");
   }
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc(TcArgs a) {
       issue_split_gemm(tmem + (uint32_t)((NE + L) * kp), Ahi, Alo, Bhi, Blo, kp, idesc);
       mma_commit(mb);
     }
-    ok = __syncthreads_and(mbar_wait(mb, phase) ? 1 : 0) != 0;  // CTA-uniform
+    ok = __syncthreads_and(mbar_wait(mb, phase, a.wait_limit) ? 1 : 0) != 0;  // CTA-uniform
     phase ^= 1;
     asm volatile("tcgen05.fence::after_thread_sync;");
   }
@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc2(TcArgs a) {
         issue_split_gemm_tk<KP>(t_u(L), tA_hi, tA_lo, B1hi, B1lo, idesc);
         mma_commit(mb);
       }
-      ok = __syncthreads_and(mbar_wait(mb, phase) ? 1 : 0) != 0;
+      ok = __syncthreads_and(mbar_wait(mb, phase, a.wait_limit) ? 1 : 0) != 0;
       phase ^= 1;
       asm volatile("tcgen05.fence::after_thread_sync;");
     }
@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc2(TcArgs a) {
         issue_split_gemm_tk<KP>(t_w(L), tA_hi, tA_lo, B2hi, B2lo, idesc);
         mma_commit(mb);
       }
-      ok = __syncthreads_and(mbar_wait(mb, phase) ? 1 : 0) != 0;
+      ok = __syncthreads_and(mbar_wait(mb, phase, a.wait_limit) ? 1 : 0) != 0;
       phase ^= 1;
       asm volatile("tcgen05.fence::after_thread_sync;");
     }
@@ -971,7 +971,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc3(TcArgs a) {
           v1b[s2] = (in && ng - 1 - n != n) ? __ldg(a.V + (long)(ng - 1 - n) * a.ncol + col) : 0.0f;
         }
       }
-      ok = __syncthreads_and(mbar_wait(mb, phase) ? 1 : 0) != 0;
+      ok = __syncthreads_and(mbar_wait(mb, phase, a.wait_limit) ? 1 : 0) != 0;
       phase ^= 1;
       asm volatile("tcgen05.fence::after_thread_sync;");
     }
@@ -1031,7 +1031,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc3(TcArgs a) {
       asm volatile("tcgen05.fence::before_thread_sync;");
       __syncthreads();
       issue2(tWe(L), tWo(L), 2);
-      ok = __syncthreads_and(mbar_wait(mb, phase) ? 1 : 0) != 0;
+      ok = __syncthreads_and(mbar_wait(mb, phase, a.wait_limit) ? 1 : 0) != 0;
       phase ^= 1;
       asm volatile("tcgen05.fence::after_thread_sync;");
     }
@@ -1193,7 +1193,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc4(TcArgs a) {
   };
   auto wait_b = [&](int w) -> bool {
     if (!bpend[w]) return true;
-    if (!mbar_wait(smem_u32(bbar + w), bph[w])) return false;   // pending: the exit waits once more
+    if (!mbar_wait(smem_u32(bbar + w), bph[w], a.wait_limit)) return false;   // pending: the exit waits once more
     bph[w] ^= 1u;
     bpend[w] = false;
     return true;
@@ -1213,7 +1213,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc4(TcArgs a) {
       mma_commit(mb);
     }
     meanwhile();             // loads of the next phase, in flight while the MMAs run
-    ok = __syncthreads_and((mbar_wait(mb, phase) && landed) ? 1 : 0) != 0;
+    ok = __syncthreads_and((mbar_wait(mb, phase, a.wait_limit) && landed) ? 1 : 0) != 0;
     phase ^= 1;
     asm volatile("tcgen05.fence::after_thread_sync;");
   };
@@ -1911,7 +1911,7 @@ __global__ void __launch_bounds__(FL_THREADS) k_flush_tc(const float* __restrict
                                                          const long* __restrict__ colbase,
                                                          const long* __restrict__ ncols,
                                                          const long* __restrict__ accoff,
-                                                         double* __restrict__ acc,
+                                                         double* __restrict__ acc, long wait_limit,
                                                          int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char sm[];
   constexpr uint32_t abytes = FL_M * FL_KC * 4, bbytes = FL_N * FL_KC * 4;
@@ -1992,7 +1992,7 @@ __global__ void __launch_bounds__(FL_THREADS) k_flush_tc(const float* __restrict
       }
       mma_commit(mb);
     }
-    ok = __syncthreads_and(mbar_wait(mb, phase) ? 1 : 0) != 0;
+    ok = __syncthreads_and(mbar_wait(mb, phase, wait_limit) ? 1 : 0) != 0;
     phase ^= 1;
     asm volatile("tcgen05.fence::after_thread_sync;");
   }
@@ -2030,7 +2030,8 @@ __global__ void __launch_bounds__(FL_THREADS) k_flush_tc(const float* __restrict
 
 cudaError_t launch_flush_tc(const float* ph, const float* cut, long ncut_total, int kb, int nvalid, int nJ,
                             int nE, const long* colbase, const long* ncols, const long* accoff,
-                            long max_cols, double* acc, int* err, cudaStream_t st) {
+                            long max_cols, double* acc, long wait_limit, int* err,
+                            cudaStream_t st) {
   const long ytiles = (max_cols + FL_M - 1) / FL_M;
   if (ytiles > 65535) return cudaErrorInvalidConfiguration;
   dim3 grid((unsigned)((2 * nE + FL_N - 1) / FL_N), (unsigned)ytiles, (unsigned)nJ);
@@ -2045,7 +2046,7 @@ cudaError_t launch_flush_tc(const float* ph, const float* cut, long ncut_total, 
   const int kn = std::min(kb, ((nvalid + FL_KC - 1) / FL_KC) * FL_KC);
   if (kn <= 0) return cudaSuccess;
   k_flush_tc<<<grid, FL_THREADS, smem, st>>>(ph, cut, ncut_total, kb, kn, 2 * nE, colbase, ncols,
-                                             accoff, acc, err);
+                                             accoff, acc, wait_limit, err);
   return cudaGetLastError();
 }
 
