@@ -410,7 +410,8 @@ int mw3_product_probabilities(mw3_ctx* ctx, double* P);
  *                as MW3_ERR_TIMEOUT, after which the context is not usable for propagation;
  *                mw3_apply_hs, mw3_lanczos and the bound-state calls return it and leave the
  *                propagation state alone. 0 makes every wait run out (the failure-detection
- *                tests).
+ *                tests); values between count in the tile-major mixed form only, the others
+ *                take them as the default.
  * Values outside a key's range return MW3_ERR_BAD_ARG. mw3_get_tuning reads a key. */
 int mw3_set_tuning(mw3_ctx* ctx, const char* key, long value);
 long mw3_get_tuning(const mw3_ctx* ctx, const char* key);

@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc(TcArgs a) {
       issue_split_gemm(tmem + (uint32_t)(L * kp), Ahi, Alo, Bhi, Blo, kp, idesc);
       mma_commit(mb);
     }
-    ok = __syncthreads_and(mbar_wait(mb, phase, a.wait_limit) ? 1 : 0) != 0;  // CTA-uniform
+    ok = __syncthreads_and(mbar_wait_full(mb, phase, a.wait_limit) ? 1 : 0) != 0;  // CTA-uniform
     phase ^= 1;
     asm volatile("tcgen05.fence::after_thread_sync;");
   }
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc(TcArgs a) {
       issue_split_gemm(tmem + (uint32_t)((NE + L) * kp), Ahi, Alo, Bhi, Blo, kp, idesc);
       mma_commit(mb);
     }
-    ok = __syncthreads_and(mbar_wait(mb, phase, a.wait_limit) ? 1 : 0) != 0;  // CTA-uniform
+    ok = __syncthreads_and(mbar_wait_full(mb, phase, a.wait_limit) ? 1 : 0) != 0;  // CTA-uniform
     phase ^= 1;
     asm volatile("tcgen05.fence::after_thread_sync;");
   }
@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc2(TcArgs a) {
         issue_split_gemm_tk<KP>(t_u(L), tA_hi, tA_lo, B1hi, B1lo, idesc);
         mma_commit(mb);
       }
-      ok = __syncthreads_and(mbar_wait(mb, phase, a.wait_limit) ? 1 : 0) != 0;
+      ok = __syncthreads_and(mbar_wait_full(mb, phase, a.wait_limit) ? 1 : 0) != 0;
       phase ^= 1;
       asm volatile("tcgen05.fence::after_thread_sync;");
     }
@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc2(TcArgs a) {
         issue_split_gemm_tk<KP>(t_w(L), tA_hi, tA_lo, B2hi, B2lo, idesc);
         mma_commit(mb);
       }
-      ok = __syncthreads_and(mbar_wait(mb, phase, a.wait_limit) ? 1 : 0) != 0;
+      ok = __syncthreads_and(mbar_wait_full(mb, phase, a.wait_limit) ? 1 : 0) != 0;
       phase ^= 1;
       asm volatile("tcgen05.fence::after_thread_sync;");
     }
@@ -971,7 +971,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc3(TcArgs a) {
           v1b[s2] = (in && ng - 1 - n != n) ? __ldg(a.V + (long)(ng - 1 - n) * a.ncol + col) : 0.0f;
         }
       }
-      ok = __syncthreads_and(mbar_wait(mb, phase, a.wait_limit) ? 1 : 0) != 0;
+      ok = __syncthreads_and(mbar_wait_full(mb, phase, a.wait_limit) ? 1 : 0) != 0;
       phase ^= 1;
       asm volatile("tcgen05.fence::after_thread_sync;");
     }
@@ -1031,7 +1031,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc3(TcArgs a) {
       asm volatile("tcgen05.fence::before_thread_sync;");
       __syncthreads();
       issue2(tWe(L), tWo(L), 2);
-      ok = __syncthreads_and(mbar_wait(mb, phase, a.wait_limit) ? 1 : 0) != 0;
+      ok = __syncthreads_and(mbar_wait_full(mb, phase, a.wait_limit) ? 1 : 0) != 0;
       phase ^= 1;
       asm volatile("tcgen05.fence::after_thread_sync;");
     }
@@ -1193,7 +1193,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc4(TcArgs a) {
   };
   auto wait_b = [&](int w) -> bool {
     if (!bpend[w]) return true;
-    if (!mbar_wait(smem_u32(bbar + w), bph[w], a.wait_limit)) return false;   // pending: the exit waits once more
+    // an expired copy stays pending: the exit waits once more
+    if (!mbar_wait_full(smem_u32(bbar + w), bph[w], a.wait_limit)) return false;
     bph[w] ^= 1u;
     bpend[w] = false;
     return true;
@@ -1213,7 +1214,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc4(TcArgs a) {
       mma_commit(mb);
     }
     meanwhile();             // loads of the next phase, in flight while the MMAs run
-    ok = __syncthreads_and((mbar_wait(mb, phase, a.wait_limit) && landed) ? 1 : 0) != 0;
+    ok = __syncthreads_and((mbar_wait_full(mb, phase, a.wait_limit) && landed) ? 1 : 0) != 0;
     phase ^= 1;
     asm volatile("tcgen05.fence::after_thread_sync;");
   };
@@ -1992,7 +1993,7 @@ __global__ void __launch_bounds__(FL_THREADS) k_flush_tc(const float* __restrict
       }
       mma_commit(mb);
     }
-    ok = __syncthreads_and(mbar_wait(mb, phase, wait_limit) ? 1 : 0) != 0;
+    ok = __syncthreads_and(mbar_wait_full(mb, phase, wait_limit) ? 1 : 0) != 0;
     phase ^= 1;
     asm volatile("tcgen05.fence::after_thread_sync;");
   }
