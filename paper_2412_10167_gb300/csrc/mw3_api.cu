@@ -2271,15 +2271,15 @@ int peek_max(const mw3_ctx* ctx) { return ctx->precision == MW3_FP64 ? kPeekMax 
 int flux_flushed(mw3_ctx* ctx) {
   const int nJ = ctx->nJ, nE = ctx->an.nE;
   if (ctx->fluxA_version == ctx->acc_version && dptr(ctx, "fluxA")) return MW3_OK;
-  const long max_ncut = *std::max_element(ctx->ncut.begin(), ctx->ncut.end());
+  const int nz = flux_chunks(ctx->ncut, nE, ctx->nsm);
   const bool mixed = ctx->precision != MW3_FP64;
   int st;
-  if ((st = dalloc(ctx, "flux_part", (size_t)flux_partial_size(nJ, nE, max_ncut) * 8)) ||
+  if ((st = dalloc(ctx, "flux_part", (size_t)nz * nJ * nE * 8)) ||
       (st = dalloc(ctx, "fluxA", (size_t)nJ * nE * 8)) ||
       (mixed && (st = dalloc(ctx, "acc32", (size_t)ctx->acc_size * 4))))
     return st;
   LK(launch_flux_reduce((const double*)dptr(ctx, "acc"), nJ, nE, (const long*)dptr(ctx, "accoff"),
-                        (const long*)dptr(ctx, "ncols"), (const long*)dptr(ctx, "ncut"), max_ncut,
+                        (const long*)dptr(ctx, "ncols"), (const long*)dptr(ctx, "ncut"), nz, ctx->nsm,
                         (double*)dptr(ctx, "flux_part"), (double*)dptr(ctx, "fluxA"),
                         mixed ? (float*)dptr(ctx, "acc32") : nullptr, ctx->stream));
   ctx->fluxA_version = ctx->acc_version;
@@ -2294,17 +2294,17 @@ int flux_peek(mw3_ctx* ctx) {
   Bufs<real> B = bufs<real>(ctx);
   const int nJ = ctx->nJ, nE = ctx->an.nE, kb = ctx->tune.kb;
   LK(launch_phases<real>(B.theta, nJ, nE, kb, ctx->ring_n, ctx->ring_n, B.d_iter, B.ph, ctx->stream));
-  const long max_ncut = *std::max_element(ctx->ncut.begin(), ctx->ncut.end());
+  const int nz = flux_chunks(ctx->ncut, nE, ctx->nsm);
   int st;
-  if ((st = dalloc(ctx, "flux_part", (size_t)flux_partial_size(nJ, nE, max_ncut) * 8))) return st;
+  if ((st = dalloc(ctx, "flux_part", (size_t)nz * nJ * nE * 8))) return st;
   if constexpr (std::is_same<real, float>::value) {
     if ((st = flux_flushed(ctx))) return st;
     LK(launch_flux_cross((const float*)dptr(ctx, "acc32"), nJ, nE, B.accoff, B.ncols, B.ncut,
-                         max_ncut, B.ph, kb, ctx->ring_n, B.cut, ctx->NC, B.colbase,
+                         nz, ctx->nsm, B.ph, kb, ctx->ring_n, B.cut, ctx->NC, B.colbase,
                          (double*)dptr(ctx, "flux_part"), (const double*)dptr(ctx, "fluxA"),
                          (double*)dptr(ctx, "flux"), ctx->stream));
   } else {
-    LK(launch_flux_reduce_peek<real>(B.acc, nJ, nE, B.accoff, B.ncols, B.ncut, max_ncut, B.ph, kb,
+    LK(launch_flux_reduce_peek<real>(B.acc, nJ, nE, B.accoff, B.ncols, B.ncut, nz, ctx->nsm, B.ph, kb,
                                      ctx->ring_n, B.cut, ctx->NC, B.colbase,
                                      (double*)dptr(ctx, "flux_part"), (double*)dptr(ctx, "flux"),
                                      ctx->stream));

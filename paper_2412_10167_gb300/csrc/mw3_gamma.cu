@@ -553,7 +553,7 @@ cudaError_t launch_dots(const real* a, const real* b, const long* J_begin, int n
 // with A rows e (real part) and nE + e (imaginary part).
 // The flux sum of Eq. total-flux per (J, E): F = sum_p Re A(p) Im B(p) - Im A(p) Re B(p) over
 // the J's cut points p (A the psi columns, B the dpsi columns of the accumulators), split over
-// chunks of kFluxChunk points so that every SM takes part (the accumulators are GBs: the
+// chunks of its points so that every SM takes part (the accumulators are GBs: the
 // reduction is one read of them), with partial sums per chunk summed in chunk order by
 // k_flux_final. PEEK: the accumulators are A + Ph Cut with the ring slots that have not been
 // flushed yet (npend <= kPeekMax) added on the fly (FP32 products summed in FP32, then added to
@@ -561,12 +561,27 @@ cudaError_t launch_dots(const real* a, const real* b, const long* J_begin, int n
 // probability read between flushes moves the accumulators once instead of three times (read
 // and write of a flush, then the read of the reduction).
 constexpr int kFluxE = 8;          // energies per CTA (the ring values of a point read once)
-constexpr long kFluxChunk = 4096;  // cut points per CTA, halved while that leaves SMs idle (down
-                                   // to 512: 40x36x20 with 64 energies had 24 CTAs of 4096)
-static long flux_chunk(int nJ, int nE, long max_ncut) {
-  long c = kFluxChunk;
-  while (c > 512 && ((max_ncut + c - 1) / c) * nJ * ((nE + kFluxE - 1) / kFluxE) < 304) c /= 2;
-  return c;
+// Cut points per CTA: 2^12, halved (down to 2^9) while one J has fewer CTAs than the part has SMs
+// (40x36x20 with 64 energies had 16 CTAs of 4096). The rule sees this J alone, so that a J has the
+// same bits alone and in a batch. A batch then has more, smaller CTAs than it needs: a read with one
+// pending slot of ten J on 40x36x20 takes 180 instead of 170 us (twelve J on 64x48x24, 200 energies:
+// 369 and 360; in FP64 807 and 914, 2840 and 2950). With twice as many CTAs per J these were 182 and 408 us, and a single J was no
+// faster (J = 10 on 64x48x24: 35 against 30 us for k_flux_cross).
+constexpr int kFluxChunkLg = 12, kFluxChunkMinLg = 9;
+static __host__ __device__ __forceinline__ int flux_chunk_lg(long np, int nE, int nsm) {
+  int lg = kFluxChunkLg;
+  const long ne = (nE + kFluxE - 1) / kFluxE;
+  while (lg > kFluxChunkMinLg && ((np + (1L << lg) - 1) >> lg) * ne < nsm) --lg;
+  return lg;
+}
+
+int flux_chunks(const std::vector<long>& ncut, int nE, int nsm) {
+  long nz = 1;
+  for (long np : ncut) {
+    const int lg = flux_chunk_lg(np, nE, nsm);
+    nz = std::max(nz, (np + (1L << lg) - 1) >> lg);
+  }
+  return (int)nz;
 }
 
 template <bool PEEK, typename real>
@@ -574,7 +589,7 @@ __global__ void __launch_bounds__(256) k_flux_partial(
     const double* __restrict__ acc, int nJ, int nE, const long* __restrict__ accoff,
     const long* __restrict__ ncols, const long* __restrict__ ncut, const real* __restrict__ ph,
     int kb, int npend, const real* __restrict__ cut, long ncut_total,
-    const long* __restrict__ colbase, long chunk, double* __restrict__ part, float* __restrict__ acc32) {
+    const long* __restrict__ colbase, int nsm, double* __restrict__ part, float* __restrict__ acc32) {
   // phase factors (real, imaginary row) per pending slot, in the ring's precision: the pending
   // terms are summed like the flush sums them (FP32 products in the mixed form; FP64 arithmetic
   // runs at 1/64 of the FP32 rate here) and added to the FP64 accumulators once
@@ -584,7 +599,12 @@ __global__ void __launch_bounds__(256) k_flux_partial(
   const int iJ = blockIdx.y;
   const int ne = min(kFluxE, nE - e0);
   const long nc = ncols[iJ], np = ncut[iJ];
-  const long p0 = (long)blockIdx.z * chunk, p1 = min(np, p0 + chunk);
+  const int lg = flux_chunk_lg(np, nE, nsm);
+  const long p0 = (long)blockIdx.z << lg, p1 = min(np, p0 + (1L << lg));
+  if (p0 >= np) {   // a J with fewer chunks than the launch has
+    if (threadIdx.x < ne) part[((long)blockIdx.z * nJ + iJ) * nE + e0 + threadIdx.x] = 0.0;
+    return;
+  }
   const double* A = acc + accoff[iJ];
   if constexpr (PEEK) {
     for (int x = threadIdx.x; x < kFluxE * 2 * kPeekMax; x += blockDim.x) {
@@ -689,14 +709,19 @@ __global__ void __launch_bounds__(256, 2) k_flux_cross(
     const float* __restrict__ acc32, int nJ, int nE, const long* __restrict__ accoff,
     const long* __restrict__ ncols, const long* __restrict__ ncut, const float* __restrict__ ph,
     int kb, int npend, const float* __restrict__ cut, long ncut_total,
-    const long* __restrict__ colbase, long chunk, double* __restrict__ part) {
+    const long* __restrict__ colbase, int nsm, double* __restrict__ part) {
   __shared__ __align__(16) float2 sph[kFluxE][NP];
   __shared__ double red[kFluxE][256];
   const int e0 = blockIdx.x * kFluxE;
   const int iJ = blockIdx.y;
   const int ne = min(kFluxE, nE - e0);
   const long nc = ncols[iJ], np = ncut[iJ];
-  const long p0 = (long)blockIdx.z * chunk, p1 = min(np, p0 + chunk);
+  const int lg = flux_chunk_lg(np, nE, nsm);
+  const long p0 = (long)blockIdx.z << lg, p1 = min(np, p0 + (1L << lg));
+  if (p0 >= np) {   // a J with fewer chunks than the launch has
+    if (threadIdx.x < ne) part[((long)blockIdx.z * nJ + iJ) * nE + e0 + threadIdx.x] = 0.0;
+    return;
+  }
   const float* A = acc32 + accoff[iJ];
   const float* cj = cut + colbase[iJ];
   for (int x = threadIdx.x; x < kFluxE * NP; x += blockDim.x) {
@@ -770,22 +795,16 @@ __global__ void k_flux_final(const double* __restrict__ part, int nz, long n,
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double s = 0.0;
+#pragma unroll 8
   for (int z = 0; z < nz; ++z) s += part[(long)z * n + i];
   out[i] = base ? base[i] + s : s;
 }
 
-long flux_partial_size(int nJ, int nE, long max_ncut) {
-  const long chunk = flux_chunk(nJ, nE, max_ncut);
-  return std::max<long>(1, (max_ncut + chunk - 1) / chunk) * nJ * nE;
-}
-
 cudaError_t launch_flux_reduce(const double* acc, int nJ, int nE, const long* accoff,
-                               const long* ncols, const long* ncut, long max_ncut, double* part,
+                               const long* ncols, const long* ncut, int nz, int nsm, double* part,
                                double* out, float* acc32, cudaStream_t st) {
-  const long chunk = flux_chunk(nJ, nE, max_ncut);
-  const int nz = (int)std::max<long>(1, (max_ncut + chunk - 1) / chunk);
   k_flux_partial<false, double><<<dim3((nE + kFluxE - 1) / kFluxE, nJ, nz), 256, 0, st>>>(
-      acc, nJ, nE, accoff, ncols, ncut, nullptr, 0, 0, nullptr, 0, nullptr, chunk, part, acc32);
+      acc, nJ, nE, accoff, ncols, ncut, nullptr, 0, 0, nullptr, 0, nullptr, nsm, part, acc32);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const long n = (long)nJ * nE;
@@ -795,15 +814,13 @@ cudaError_t launch_flux_reduce(const double* acc, int nJ, int nE, const long* ac
 
 template <typename real>
 cudaError_t launch_flux_reduce_peek(const double* acc, int nJ, int nE, const long* accoff,
-                                    const long* ncols, const long* ncut, long max_ncut,
+                                    const long* ncols, const long* ncut, int nz, int nsm,
                                     const real* ph, int kb, int npend, const real* cut,
                                     long ncut_total, const long* colbase, double* part,
                                     double* out, cudaStream_t st) {
   if (npend < 0 || npend > kPeekMax) return cudaErrorInvalidValue;
-  const long chunk = flux_chunk(nJ, nE, max_ncut);
-  const int nz = (int)std::max<long>(1, (max_ncut + chunk - 1) / chunk);
   k_flux_partial<true, real><<<dim3((nE + kFluxE - 1) / kFluxE, nJ, nz), 256, 0, st>>>(
-      acc, nJ, nE, accoff, ncols, ncut, ph, kb, npend, cut, ncut_total, colbase, chunk, part, nullptr);
+      acc, nJ, nE, accoff, ncols, ncut, ph, kb, npend, cut, ncut_total, colbase, nsm, part, nullptr);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const long n = (long)nJ * nE;
@@ -812,17 +829,15 @@ cudaError_t launch_flux_reduce_peek(const double* acc, int nJ, int nE, const lon
 }
 
 cudaError_t launch_flux_cross(const float* acc32, int nJ, int nE, const long* accoff,
-                              const long* ncols, const long* ncut, long max_ncut, const float* ph,
+                              const long* ncols, const long* ncut, int nz, int nsm, const float* ph,
                               int kb, int npend, const float* cut, long ncut_total,
                               const long* colbase, double* part, const double* fluxA, double* out,
                               cudaStream_t st) {
   if (npend < 0 || npend > kPeekMaxX || npend > kb) return cudaErrorInvalidValue;
-  const long chunk = flux_chunk(nJ, nE, max_ncut);
-  const int nz = (int)std::max<long>(1, (max_ncut + chunk - 1) / chunk);
   const dim3 grid((nE + kFluxE - 1) / kFluxE, nJ, nz);
 #define CROSS(NP)                                                                                       \
   k_flux_cross<NP><<<grid, 256, 0, st>>>(acc32, nJ, nE, accoff, ncols, ncut, ph, kb, npend, cut, \
-                                         ncut_total, colbase, chunk, part)
+                                         ncut_total, colbase, nsm, part)
   if (npend <= 4) CROSS(4);
   else if (npend <= 8) CROSS(8);
   else if (npend <= 12) CROSS(12);
@@ -913,7 +928,7 @@ cudaError_t launch_channel_probs(const double* acc, const ChanTable& t, const Ch
 
 #define MW3_INST(real)                                                                        \
   template cudaError_t launch_flux_reduce_peek<real>(const double*, int, int, const long*,      \
-                                                     const long*, const long*, long, const real*, \
+                                                     const long*, const long*, int, int, const real*, \
                                                      int, int, const real*, long, const long*,   \
                                                      double*, double*, cudaStream_t);            \
   template cudaError_t launch_gamma_forward<real>(const real*, real*, const real*,            \
