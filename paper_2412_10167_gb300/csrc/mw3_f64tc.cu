@@ -425,13 +425,9 @@ cudaError_t launch_inst(const F64Args& a, cudaStream_t st) {
   static_assert(sm <= 227 * 1024, "shared memory of the FP64 angular step");
   static_assert(kSlices * (KH / 2) + kLevels * f64tc_chunk(KH) <= 512, "tensor memory of the FP64 angular step");
   static_assert((long)kSlices * KH * 16384 < (1L << 24), "level sums exact in FP32");
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(k_angular_f64<KH, NE>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static OncePerDevice attr;
+  const cudaError_t e = allow_smem(attr, k_angular_f64<KH, NE>, sm);
+  if (e != cudaSuccess) return e;
   const long total = (long)a.ngroups * a.ntiles;
   const unsigned grid = (unsigned)std::min<long>(a.nsm, total);
   k_angular_f64<KH, NE><<<grid, kThreads, sm, st>>>(a);

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/mw3.h"
+#include "mw3_device.h"
 #include "mw3_wigner.h"
 
 namespace mw3 {

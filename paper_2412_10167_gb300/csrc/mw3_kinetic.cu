@@ -371,13 +371,9 @@ cudaError_t launch_kinetic_rows(const real* q, real* t, long nrows, const FFTPla
   if (kinetic_rows_fixed<real>(plan.N, q, t, nrows, tw, ph, lam, pairs, blocks, ng, nr, st, &err))
     return err;
   const size_t sm = kinetic_smem<real>(plan.N, pairs);
-  static bool attr_set[2] = {false, false};
-  const int slot = sizeof(real) == 8 ? 1 : 0;
-  if (!attr_set[slot]) {
-    cudaFuncSetAttribute(k_kinetic_rows<real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         227 * 1024);
-    attr_set[slot] = true;
-  }
+  static OncePerDevice attr;
+  err = allow_smem(attr, k_kinetic_rows<real>, 227 * 1024);
+  if (err != cudaSuccess) return err;
   const long npairs = (nrows + 1) / 2;
   const unsigned grid = (unsigned)((npairs + pairs - 1) / pairs);
   k_kinetic_rows<real><<<grid, 256, sm, st>>>(q, t, nrows, plan,
@@ -407,13 +403,9 @@ cudaError_t launch_kinetic_cols(const real* q, real* t, long nplanes, int nr, in
                                cut_slot, blocks, ncut_J, m_inf, qcol, st, &err))
     return err;
   const size_t sm = kinetic_smem<real>(plan.N, ctile / 2);
-  static bool attr_set[2] = {false, false};
-  const int slot = sizeof(real) == 8 ? 1 : 0;
-  if (!attr_set[slot]) {
-    cudaFuncSetAttribute(k_kinetic_cols<real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         227 * 1024);
-    attr_set[slot] = true;
-  }
+  static OncePerDevice attr;
+  err = allow_smem(attr, k_kinetic_cols<real>, 227 * 1024);
+  if (err != cudaSuccess) return err;
   dim3 grid((unsigned)((NR + ctile - 1) / ctile), (unsigned)nplanes);
   k_kinetic_cols<real><<<grid, 256, sm, st>>>(q, t, nr, NR, plan,
                                               static_cast<const cpx<real>*>(tw),

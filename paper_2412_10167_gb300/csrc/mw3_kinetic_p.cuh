@@ -416,13 +416,7 @@ __global__ void __launch_bounds__(kPThreads, (kMinCtas<T, N1, N2>)) k_cols_p(
 
 // log2 of the pairs per tile: the most, halved (down to 4) while fewer tiles than SMs result.
 inline int tile_lg(int most, long pairs_per_line, long lines) {
-  static int nsm = 0;
-  if (!nsm) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    nsm = std::max(nsm, 1);
-  }
+  const int nsm = sm_count();
   int lg = most == 32 ? 5 : 4;
   while (lg > 2 && ((pairs_per_line + (1 << lg) - 1) >> lg) * lines < nsm) --lg;
   return lg;
@@ -433,17 +427,15 @@ cudaError_t rows_p(const T* q, T* t, long nrows, const void* tw, const void* ph,
                    const DevBlock* blocks, int ng, int nr, cudaStream_t st) {
   constexpr size_t sm = rows_smem<T, N1, N2>();
   static_assert(sm <= 227 * 1024, "shared memory of the row kernel");
-  static int grid_max = 0;
-  if (!grid_max) {
-    const cudaError_t e = cudaFuncSetAttribute(k_rows_p<T, N1, N2>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    int dev = 0, nsm = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_rows_p<T, N1, N2>, kPThreads, sm);
-    grid_max = std::max(nsm, 1) * std::max(per, 1);
-  }
+  static OncePerDevice attr;
+  static IntPerDevice per;
+  const cudaError_t e = allow_smem(attr, k_rows_p<T, N1, N2>, sm);
+  if (e != cudaSuccess) return e;
+  const int grid_max = sm_count() * per.get(current_device(), [&] {
+    int n = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_rows_p<T, N1, N2>, kPThreads, sm);
+    return std::max(n, 1);
+  });
   const int lg = tile_lg(kPairs<T, N1 * N2>, nrows / 2, 1);
   const long ntile = ((nrows + 1) / 2 + (1 << lg) - 1) >> lg;
   k_rows_p<T, N1, N2><<<(unsigned)std::min<long>(ntile, grid_max), kPThreads, sm, st>>>(
@@ -457,13 +449,9 @@ cudaError_t cols_p(const T* q, T* t, long nplanes, int NR, const void* tw, const
                    const DevBlock* blocks, const int* ncut_J, int m_inf, T* qcol, cudaStream_t st) {
   constexpr size_t sm = cols_smem<T, N1, N2>();
   static_assert(sm <= 227 * 1024, "shared memory of the column kernel");
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(k_cols_p<T, N1, N2>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static OncePerDevice attr;
+  const cudaError_t e = allow_smem(attr, k_cols_p<T, N1, N2>, sm);
+  if (e != cudaSuccess) return e;
   const int lg = tile_lg(kPairs<T, N1 * N2>, NR / 2, nplanes);
   dim3 grid((unsigned)((NR / 2 + (1 << lg) - 1) >> lg), (unsigned)nplanes);
   k_cols_p<T, N1, N2><<<grid, kPThreads, sm, st>>>(q, t, NR, static_cast<const cpx<T>*>(tw),

@@ -185,11 +185,9 @@ size_t smem_rows(int N, int P) {
 template <typename T, int N>
 cudaError_t rows_inst(const T* q, T* t, long nrows, const void* tw, const void* ph, const T* lam,
                       int P, const DevBlock* blocks, int ng, int nr, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_rows_t<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    attr = true;
-  }
+  static OncePerDevice attr;
+  const cudaError_t ea = allow_smem(attr, k_rows_t<T, N>, 227 * 1024);
+  if (ea != cudaSuccess) return ea;
   const long npairs = (nrows + 1) / 2;
   const unsigned grid = (unsigned)((npairs + P - 1) / P);
   k_rows_t<T, N><<<grid, 256, smem_rows<T>(N, P), st>>>(
@@ -203,11 +201,9 @@ cudaError_t cols_inst(const T* q, T* t, long nplanes, int NR, const void* tw, co
                       const T* lam, int C, int ng, const T* wpsi, const T* wdpsi, T* cut,
                       const DevBlock* blocks, const int* ncut_J, int m_inf, T* qcol,
                       cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_cols_t<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    attr = true;
-  }
+  static OncePerDevice attr;
+  const cudaError_t ea = allow_smem(attr, k_cols_t<T, N>, 227 * 1024);
+  if (ea != cudaSuccess) return ea;
   const size_t sm = smem_rows<T>(N, C / 2) + sizeof(T) * 8 * (size_t)C;
   dim3 grid((unsigned)((NR + C - 1) / C), (unsigned)nplanes);
   k_cols_t<T, N><<<grid, 256, sm, st>>>(q, t, NR, static_cast<const cpx<T>*>(tw),

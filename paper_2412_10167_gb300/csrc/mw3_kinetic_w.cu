@@ -396,17 +396,11 @@ bool rows_w(const T* q, T* t, long nrows, const void* tw, const void* ph, const 
   } else {
     constexpr int N = 32 * R;
     const size_t sm = ((sizeof(WTables<T, R>) + 15) / 16) * 16 + 2 * 16 * (size_t)N * sizeof(T);
-    static bool attr = false;
-    static int nsm = 0;
-    if (!attr) {
-      cudaFuncSetAttribute(k_rows_w<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      int dev = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-      attr = true;
-    }
+    static OncePerDevice attr;
+    *err = allow_smem(attr, k_rows_w<T, R>, sm);
+    if (*err != cudaSuccess) return true;
     const long nrb = (nrows + 15) / 16;
-    const unsigned grid = (unsigned)std::min<long>(nrb, (long)std::max(nsm, 1) * kMinBlocks<T, R>);
+    const unsigned grid = (unsigned)std::min<long>(nrb, (long)sm_count() * kMinBlocks<T, R>);
     k_rows_w<T, R><<<grid, 256, sm, st>>>(q, t, nrows, static_cast<const cpx<T>*>(tw),
                                           static_cast<const cpx<T>*>(ph), lam, blocks, ng, nr);
     *err = cudaGetLastError();
@@ -421,12 +415,9 @@ bool cols_wc(const T* q, T* t, long nplanes, int NR, const void* tw, const void*
              cudaError_t* err) {
   constexpr int N = 32 * R;
   const size_t sm = sizeof(WTables<T, R>) + sizeof(T) * ((size_t)N * (C + 1) + 8 * (size_t)C);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_cols_w<T, R, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         227 * 1024);
-    attr = true;
-  }
+  static OncePerDevice attr;
+  *err = allow_smem(attr, k_cols_w<T, R, C>, 227 * 1024);
+  if (*err != cudaSuccess) return true;
   dim3 grid((unsigned)((NR + C - 1) / C), (unsigned)nplanes);
   k_cols_w<T, R, C><<<grid, 256, sm, st>>>(q, t, NR, static_cast<const cpx<T>*>(tw),
                                            static_cast<const cpx<T>*>(ph), lam, ng, wpsi, wdpsi,
@@ -649,19 +640,17 @@ bool rows_hw(const float* q, float* t, long nrows, const void* tw, const void* p
              cudaError_t* err) {
   constexpr int N = 16 * N1;
   const size_t sm = ((sizeof(HwTables<N1>) + 15) / 16) * 16 + 2 * 32 * (size_t)(N + 8) * sizeof(float);
-  static bool attr = false;
-  static int nsm = 0, per_sm = 1;
-  if (!attr) {
-    cudaFuncSetAttribute(k_rows_hw<N1, SHFL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rows_hw<N1, SHFL>, 256, sm);
-    per_sm = std::max(per_sm, 1);
-    attr = true;
-  }
+  static OncePerDevice attr;
+  static IntPerDevice per;
+  *err = allow_smem(attr, k_rows_hw<N1, SHFL>, sm);
+  if (*err != cudaSuccess) return true;
+  const int per_sm = per.get(current_device(), [&] {
+    int n = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_rows_hw<N1, SHFL>, 256, sm);
+    return std::max(n, 1);
+  });
   const long nrb = (nrows + 31) / 32;
-  const unsigned grid = (unsigned)std::min<long>(nrb, (long)std::max(nsm, 1) * per_sm);
+  const unsigned grid = (unsigned)std::min<long>(nrb, (long)sm_count() * per_sm);
   k_rows_hw<N1, SHFL><<<grid, 256, sm, st>>>(q, t, nrows, static_cast<const cpx<float>*>(tw),
                                        static_cast<const cpx<float>*>(ph), lam, blocks, ng, nr);
   *err = cudaGetLastError();
@@ -675,11 +664,9 @@ bool cols_hw(const float* q, float* t, long nplanes, int NR, const void* tw, con
              cudaError_t* err) {
   constexpr int N = 16 * N1;
   const size_t sm = sizeof(HwTables<N1>) + sizeof(float) * ((size_t)N * 33 + 8 * 32);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_cols_hw<N1, SHFL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    attr = true;
-  }
+  static OncePerDevice attr;
+  *err = allow_smem(attr, k_cols_hw<N1, SHFL>, sm);
+  if (*err != cudaSuccess) return true;
   dim3 grid((unsigned)((NR + 31) / 32), (unsigned)nplanes);
   k_cols_hw<N1, SHFL><<<grid, 256, sm, st>>>(q, t, NR, static_cast<const cpx<float>*>(tw),
                                        static_cast<const cpx<float>*>(ph), lam, ng, wpsi, wdpsi,

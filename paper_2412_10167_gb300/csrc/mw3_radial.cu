@@ -228,10 +228,13 @@ bool radial_launch(const float* q, float* t, long nplanes, const void* twR, cons
   if constexpr (!S::valid) {
     return false;
   } else {
-    static int ok = -1;   // the cluster shape fits on this device
-    if (ok < 0) {
-      cudaFuncSetAttribute(k_radial_hw<N1R, N1r, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)S::smem);
+    static OncePerDevice attr;
+    static IntPerDevice fits;   // 1: the cluster shape fits on this device, 2: it does not
+    const bool ok = fits.get(current_device(), [&] {
+      if (allow_smem(attr, k_radial_hw<N1R, N1r, CS>, S::smem) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 2;
+      }
       cudaLaunchConfig_t cfg{};
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeClusterDimension;
@@ -246,9 +249,9 @@ bool radial_launch(const float* q, float* t, long nplanes, const void* twR, cons
       int nclusters = 0;
       const cudaError_t e =
           cudaOccupancyMaxActiveClusters(&nclusters, k_radial_hw<N1R, N1r, CS>, &cfg);
-      ok = (e == cudaSuccess && nclusters > 0) ? 1 : 0;
       (void)cudaGetLastError();
-    }
+      return e == cudaSuccess && nclusters > 0 ? 1 : 2;
+    }) == 1;
     if (!ok) return false;
     if (q == nullptr) return true;   // query: the shape is built and fits on this device
     cudaLaunchConfig_t cfg{};

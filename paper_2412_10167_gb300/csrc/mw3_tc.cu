@@ -2037,11 +2037,9 @@ cudaError_t launch_flush_tc(const float* ph, const float* cut, long ncut_total, 
   if (ytiles > 65535) return cudaErrorInvalidConfiguration;
   dim3 grid((unsigned)((2 * nE + FL_N - 1) / FL_N), (unsigned)ytiles, (unsigned)nJ);
   const size_t smem = 2 * (size_t)FL_M * FL_KC * 4 + 2 * (size_t)FL_N * FL_KC * 4 + 64;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_flush_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr = true;
-  }
+  static OncePerDevice attr;
+  const cudaError_t ea = allow_smem(attr, k_flush_tc, smem);
+  if (ea != cudaSuccess) return ea;
   // ring slots past the valid ones carry zero phases: multiply the valid ones only (K rounded up
   // to the chunk FL_KC); ph rows keep the stride kb
   const int kn = std::min(kb, ((nvalid + FL_KC - 1) / FL_KC) * FL_KC);
@@ -2057,12 +2055,9 @@ size_t angular_tc_smem(int kp) {
 
 template <int KP, int NE>
 static cudaError_t launch_tc_inst(const TcArgs& args, dim3 grid, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_angular_tc<KP, NE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         227 * 1024);
-    attr = true;
-  }
+  static OncePerDevice attr;
+  const cudaError_t ea = allow_smem(attr, k_angular_tc<KP, NE>, 227 * 1024);
+  if (ea != cudaSuccess) return ea;
   k_angular_tc<KP, NE><<<grid, TC_THREADS, angular_tc_smem(KP), st>>>(args);
   return cudaGetLastError();
 }
@@ -2072,12 +2067,9 @@ static cudaError_t launch_tc2_inst(const TcArgs& args, cudaStream_t st) {
   if constexpr (NE == 2 && (2 + 2 + 1) * KP > 512) {
     return cudaErrorInvalidValue;   // tensor-memory columns: 5 kp for two states
   } else {
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(k_angular_tc2<KP, NE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           227 * 1024);
-      attr = true;
-    }
+    static OncePerDevice attr;
+    const cudaError_t ea = allow_smem(attr, k_angular_tc2<KP, NE>, 227 * 1024);
+    if (ea != cudaSuccess) return ea;
     const long total = (long)args.ngroups * args.ntiles;
     const unsigned grid = (unsigned)std::min<long>(total, args.nsm);
     k_angular_tc2<KP, NE><<<grid, TC_THREADS, tc2_smem<KP>(), st>>>(args);
@@ -2101,12 +2093,9 @@ static cudaError_t launch_tc2_ne(const TcArgs& a, cudaStream_t st) {
 
 template <int KH, int NE>
 static cudaError_t launch_tc3_inst(const TcArgs& args, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_angular_tc3<KH, NE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         227 * 1024);
-    attr = true;
-  }
+  static OncePerDevice attr;
+  const cudaError_t ea = allow_smem(attr, k_angular_tc3<KH, NE>, 227 * 1024);
+  if (ea != cudaSuccess) return ea;
   const long total = (long)args.ngroups * args.ntiles;
   const unsigned grid = (unsigned)std::min<long>(total, args.nsm);
   k_angular_tc3<KH, NE><<<grid, TC_THREADS, tc3_smem<KH>(), st>>>(args);
@@ -2125,12 +2114,9 @@ static cudaError_t launch_tc3_ne(const TcArgs& a, cudaStream_t st) {
 
 template <int KH>
 static cudaError_t launch_tc4_inst(const TcArgs& args, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_angular_tc4<KH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         227 * 1024);
-    attr = true;
-  }
+  static OncePerDevice attr;
+  const cudaError_t ea = allow_smem(attr, k_angular_tc4<KH>, 227 * 1024);
+  if (ea != cudaSuccess) return ea;
   const long total = (long)args.ngroups * args.ntiles;
   const unsigned grid = (unsigned)std::min<long>(total, args.nsm);
   k_angular_tc4<KH><<<grid, TC_THREADS, tc4_smem<KH>(), st>>>(args);
@@ -2148,12 +2134,9 @@ static cudaError_t launch_tc4(const TcArgs& a, cudaStream_t st) {
 
 template <int KH, bool TMA>
 static cudaError_t launch_tc5_tma(const TcArgs& args, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_angular_tc5<KH, TMA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         227 * 1024);
-    attr = true;
-  }
+  static OncePerDevice attr;
+  const cudaError_t ea = allow_smem(attr, k_angular_tc5<KH, TMA>, 227 * 1024);
+  if (ea != cudaSuccess) return ea;
   const long total = (long)args.ngroups * args.ntiles;
   const unsigned grid = (unsigned)std::min<long>(total, args.nsm);
   k_angular_tc5<KH, TMA><<<grid, TC_THREADS, tc5_smem<KH>(), st>>>(args);
