@@ -409,9 +409,9 @@ int mw3_product_probabilities(mw3_ctx* ctx, double* P);
  *                probability read or checkpoint that flushes pending iterations) returns it
  *                as MW3_ERR_TIMEOUT, after which the context is not usable for propagation;
  *                mw3_apply_hs, mw3_lanczos and the bound-state calls return it and leave the
- *                propagation state alone. 0 makes every wait run out (the failure-detection
- *                tests); values between count in the tile-major mixed form only, the others
- *                take them as the default.
+ *                propagation state alone. 0 is for the failure-detection tests: every wait of
+ *                the tile-major and FP64 forms runs out, the other forms and the flush report
+ *                one that did; other values bound the waits of the former two.
  * Values outside a key's range return MW3_ERR_BAD_ARG. mw3_get_tuning reads a key. */
 int mw3_set_tuning(mw3_ctx* ctx, const char* key, long value);
 long mw3_get_tuning(const mw3_ctx* ctx, const char* key);

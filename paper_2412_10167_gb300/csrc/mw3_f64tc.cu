@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_angular_f64(const __grid_consta
           }
           mma_commit(mb);
         }
-        ok = __syncthreads_and(mbar_wait_full(mb, phase, a.wait_limit) ? 1 : 0) != 0;
+        ok = __syncthreads_and(mbar_wait(mb, phase, a.wait_limit) ? 1 : 0) != 0;
         phase ^= 1;
         asm volatile("tcgen05.fence::after_thread_sync;");
         issue_b(kb + 2);

@@ -312,8 +312,12 @@ struct TcArgs {
   float* out;           // mode 1: H_s c
   double* npart;        // [group][tile] sums of squares of c_(k+1)
   int* err;             // set on a wait that timed out
-  long wait_limit;      // polls of a bounded wait (the wait for the MMAs of an expired phase
-                        // before tensor memory is freed keeps 2^22)
+  // polls of a bounded wait in the tile-major form (the wait for the MMAs of an expired phase before
+  // tensor memory is freed keeps 2^22). The other mixed forms and the flush keep the compile-time
+  // bound and take 0 as expired when the CTA ends: with a run-time bound, or a test for 0 at every
+  // wait, the loads in flight around the wait no longer fit in registers (512x384x180, 32 iterations:
+  // 47.4 -> 52.2 ms; flush on 256x192x96 3.67 -> 3.85 ms).
+  long wait_limit;
   float erot, alpha, beta;
   long ncol, npts;
   int ng, kp, NR, nelec, mode, ntiles, tmem_cols;
@@ -362,7 +366,7 @@ struct F64Args {
   double* out;                // mode 1: H_s c
   double* npart;              // [group][tile] sums of squares of c_(k+1)
   int* err;                   // set on a wait that timed out
-  long wait_limit;            // polls of a bounded wait (as in TcArgs)
+  long wait_limit;            // polls of a bounded wait
   double alpha, beta;
   long ncol, npts;
   int ng, kh, NR, nr, nelec, mode, ntiles, ngroups, nsm;

@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc(TcArgs a) {
       issue_split_gemm(tmem + (uint32_t)(L * kp), Ahi, Alo, Bhi, Blo, kp, idesc);
       mma_commit(mb);
     }
-    ok = __syncthreads_and(mbar_wait_full(mb, phase, a.wait_limit) ? 1 : 0) != 0;  // CTA-uniform
+    ok = __syncthreads_and(mbar_wait(mb, phase) ? 1 : 0) != 0;  // CTA-uniform
     phase ^= 1;
     asm volatile("tcgen05.fence::after_thread_sync;");
   }
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc(TcArgs a) {
       issue_split_gemm(tmem + (uint32_t)((NE + L) * kp), Ahi, Alo, Bhi, Blo, kp, idesc);
       mma_commit(mb);
     }
-    ok = __syncthreads_and(mbar_wait_full(mb, phase, a.wait_limit) ? 1 : 0) != 0;  // CTA-uniform
+    ok = __syncthreads_and(mbar_wait(mb, phase) ? 1 : 0) != 0;  // CTA-uniform
     phase ^= 1;
     asm volatile("tcgen05.fence::after_thread_sync;");
   }
@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc(TcArgs a) {
     double s = 0;
     for (int w2 = 0; w2 < TC_THREADS / 32; ++w2) s += red[w2];
     if (a.npart) a.npart[(long)g * a.ntiles + tile] = s;
-    if (!ok) atomicExch(a.err, 1);
+    if (!ok || a.wait_limit <= 0) atomicExch(a.err, 1);
   }
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;");
@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc2(TcArgs a) {
         issue_split_gemm_tk<KP>(t_u(L), tA_hi, tA_lo, B1hi, B1lo, idesc);
         mma_commit(mb);
       }
-      ok = __syncthreads_and(mbar_wait_full(mb, phase, a.wait_limit) ? 1 : 0) != 0;
+      ok = __syncthreads_and(mbar_wait(mb, phase) ? 1 : 0) != 0;
       phase ^= 1;
       asm volatile("tcgen05.fence::after_thread_sync;");
     }
@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc2(TcArgs a) {
         issue_split_gemm_tk<KP>(t_w(L), tA_hi, tA_lo, B2hi, B2lo, idesc);
         mma_commit(mb);
       }
-      ok = __syncthreads_and(mbar_wait_full(mb, phase, a.wait_limit) ? 1 : 0) != 0;
+      ok = __syncthreads_and(mbar_wait(mb, phase) ? 1 : 0) != 0;
       phase ^= 1;
       asm volatile("tcgen05.fence::after_thread_sync;");
     }
@@ -672,7 +672,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc2(TcArgs a) {
       if (a.npart) a.npart[(long)g * a.ntiles + tile] = s2;
     }
   }
-  if (!ok && tid == 0) atomicExch(a.err, 1);
+  if ((!ok || a.wait_limit <= 0) && tid == 0) atomicExch(a.err, 1);
   drain_expired(ok, mb, phase ^ 1u);   // ok is CTA-uniform; the failed wait toggled phase
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
@@ -971,7 +971,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc3(TcArgs a) {
           v1b[s2] = (in && ng - 1 - n != n) ? __ldg(a.V + (long)(ng - 1 - n) * a.ncol + col) : 0.0f;
         }
       }
-      ok = __syncthreads_and(mbar_wait_full(mb, phase, a.wait_limit) ? 1 : 0) != 0;
+      ok = __syncthreads_and(mbar_wait(mb, phase) ? 1 : 0) != 0;
       phase ^= 1;
       asm volatile("tcgen05.fence::after_thread_sync;");
     }
@@ -1031,7 +1031,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc3(TcArgs a) {
       asm volatile("tcgen05.fence::before_thread_sync;");
       __syncthreads();
       issue2(tWe(L), tWo(L), 2);
-      ok = __syncthreads_and(mbar_wait_full(mb, phase, a.wait_limit) ? 1 : 0) != 0;
+      ok = __syncthreads_and(mbar_wait(mb, phase) ? 1 : 0) != 0;
       phase ^= 1;
       asm volatile("tcgen05.fence::after_thread_sync;");
     }
@@ -1111,7 +1111,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc3(TcArgs a) {
     }
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
-  if (!ok && tid == 0) atomicExch(a.err, 1);
+  if ((!ok || a.wait_limit <= 0) && tid == 0) atomicExch(a.err, 1);
   drain_expired(ok, mb, phase ^ 1u);   // ok is CTA-uniform; the failed wait toggled phase
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
@@ -1194,7 +1194,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc4(TcArgs a) {
   auto wait_b = [&](int w) -> bool {
     if (!bpend[w]) return true;
     // an expired copy stays pending: the exit waits once more
-    if (!mbar_wait_full(smem_u32(bbar + w), bph[w], a.wait_limit)) return false;
+    if (!mbar_wait(smem_u32(bbar + w), bph[w])) return false;
     bph[w] ^= 1u;
     bpend[w] = false;
     return true;
@@ -1214,7 +1214,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc4(TcArgs a) {
       mma_commit(mb);
     }
     meanwhile();             // loads of the next phase, in flight while the MMAs run
-    ok = __syncthreads_and((mbar_wait_full(mb, phase, a.wait_limit) && landed) ? 1 : 0) != 0;
+    ok = __syncthreads_and((mbar_wait(mb, phase) && landed) ? 1 : 0) != 0;
     phase ^= 1;
     asm volatile("tcgen05.fence::after_thread_sync;");
   };
@@ -1381,7 +1381,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_angular_tc4(TcArgs a) {
   }
   for (int w = 0; w < 2; ++w)   // no copy may still be writing shared memory when the CTA ends
     if (bpend[w]) (void)mbar_wait(smem_u32(bbar + w), bph[w]);
-  if (!ok && tid == 0) atomicExch(a.err, 1);
+  if ((!ok || a.wait_limit <= 0) && tid == 0) atomicExch(a.err, 1);
   drain_expired(ok, mb, phase ^ 1u);   // ok is CTA-uniform; the failed wait toggled phase
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
@@ -1993,7 +1993,7 @@ __global__ void __launch_bounds__(FL_THREADS) k_flush_tc(const float* __restrict
       }
       mma_commit(mb);
     }
-    ok = __syncthreads_and(mbar_wait_full(mb, phase, wait_limit) ? 1 : 0) != 0;
+    ok = __syncthreads_and(mbar_wait(mb, phase) ? 1 : 0) != 0;
     phase ^= 1;
     asm volatile("tcgen05.fence::after_thread_sync;");
   }
@@ -2017,9 +2017,8 @@ __global__ void __launch_bounds__(FL_THREADS) k_flush_tc(const float* __restrict
         if (p < nE2) accJ[(long)p * nc] = o[j] + (double)v[j];
       }
     }
-  } else if (tid == 0) {
-    atomicExch(err, 1);
   }
+  if ((!ok || wait_limit <= 0) && tid == 0) atomicExch(err, 1);
   drain_expired(ok, mb, phase ^ 1u);   // ok is CTA-uniform; the failed wait toggled phase
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();

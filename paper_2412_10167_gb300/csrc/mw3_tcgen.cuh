@@ -54,14 +54,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, long l
   return false;
 }
 
-// The same with two limits only: 0 (the wait runs out at once, as the failure tests want it) and
-// the full one. The bound stays a compile-time constant: with a run-time one the loads in flight
-// around the wait no longer fitted in registers (streamed angular step of 512x384x180: 240 bytes
-// of spills, 32 iterations 47.4 -> 52.2 ms; with this form no instance of it spills).
-__device__ __forceinline__ bool mbar_wait_full(uint32_t mbar, uint32_t parity, long limit) {
-  return limit > 0 && mbar_wait(mbar, parity);
-}
-
 // After a bounded wait expired, the MMAs committed to that barrier phase may still be
 // running and writing tensor memory. Before a CTA releases its tensor memory it waits for
 // that same phase once more, again bounded: the columns are freed only after the MMAs that

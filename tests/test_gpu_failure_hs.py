@@ -1,9 +1,8 @@
 """Expired waits outside mw3_propagate, without a GPU fault.
 
-The bounded mbarrier waits of the tensor-core angular steps (every form, FP64 and mixed) and of
-the flush that a probability read may start are cut to zero polls, so that all of them run out.
-The call that started the work has to say so: its results come from tiles that were never
-written. An H_s application does not touch the propagation, which goes on as if nothing happened.
+With tc_wait_limit 0 the bounded mbarrier waits of the tile-major and of the FP64 angular step run out
+at once (the other forms and the flush report one that did). The call that started the work has to say
+so: after a wait that ran out its results come from tiles that were never written. An H_s application does not touch the propagation, which goes on as if nothing happened.
 """
 import numpy as np
 import pytest
