@@ -277,8 +277,7 @@ struct mw3_mlp {
   long ld = 0;
   double* lossp = nullptr;
   long lossp_cap = 0;
-  int* tc_err = nullptr;             // see MlpArgs::err
-  long wait_limit = 1L << 22;
+  int* tc_err = nullptr;
   int nsm = 152;
   std::string err;
 };
@@ -400,7 +399,6 @@ mw3::MlpArgs tc_args(const mw3_mlp* net, const float* X, const float* y, const i
   a.tpart = net->tpart;
   a.pstride = (net->nparam + 3) / 4 * 4;
   a.err = net->tc_err;
-  a.wait_limit = net->wait_limit;
   return a;
 }
 
@@ -444,19 +442,14 @@ mw3::MlpUpdate tc_update(const mw3_mlp* net) {
   u.shape = tc_shape(net);
   u.Wf = net->Wf;
   u.Wb = net->Wb;
-  u.err = net->tc_err;
   return u;
 }
 
-// After the stream is drained: did a bounded wait of the tensor-core kernels run out? The word is
-// cleared for the next call; `updates` (may be null) is the number of updates made since it was zeroed.
-int tc_check(mw3_mlp* net, int* updates = nullptr) {
-  int e[2] = {0, 0};
-  MCK(cudaMemcpy(e, net->tc_err, sizeof(e), cudaMemcpyDeviceToHost));
-  if (updates) *updates = e[1];
-  if (!e[0]) return MW3_OK;
-  MCK(cudaMemset(net->tc_err, 0, sizeof(int)));
-  return mfail(net, MW3_ERR_TIMEOUT, "network kernels: an mbarrier wait timed out");
+// After the stream is drained: did a bounded wait of the tensor-core kernels run out?
+int tc_check(mw3_mlp* net) {
+  int e = 0;
+  MCK(cudaMemcpy(&e, net->tc_err, sizeof(int), cudaMemcpyDeviceToHost));
+  return e ? mfail(net, MW3_ERR_TIMEOUT, "network kernels: an mbarrier wait timed out") : MW3_OK;
 }
 
 dim3 tgrid(int M, int N, int nsplit = 1) {
@@ -560,10 +553,10 @@ int create_tc(mw3_mlp* net) {
   const size_t bytes = std::max<size_t>((size_t)(net->depth - 1) * net->wp * net->wp * 2, 16);
   MCK(cudaMalloc(&net->Wf, bytes));
   MCK(cudaMalloc(&net->Wb, bytes));
-  MCK(cudaMalloc(&net->tc_err, 2 * sizeof(int)));
+  MCK(cudaMalloc(&net->tc_err, sizeof(int)));
   MCK(cudaMemset(net->Wf, 0, bytes));
   MCK(cudaMemset(net->Wb, 0, bytes));
-  MCK(cudaMemset(net->tc_err, 0, 2 * sizeof(int)));
+  MCK(cudaMemset(net->tc_err, 0, sizeof(int)));
   return MW3_OK;
 }
 
@@ -775,11 +768,6 @@ int mw3_mlp_train(mw3_mlp* net, const float* X, const float* y, long n, int epoc
   double* dloss = nullptr;
   MCK(cudaMalloc(&dloss, steps_max * sizeof(double)));
   std::vector<double> hloss(steps_max);
-  const long step0 = net->step;
-  if (net->wp && cudaMemset(net->tc_err + 1, 0, sizeof(int)) != cudaSuccess) {
-    cudaFree(dloss);
-    return mfail(net, MW3_ERR_CUDA, "mw3_mlp_train: update counter");
-  }
   for (int ep = 0; ep < epochs; ++ep) {
     std::shuffle(perm.begin(), perm.end(), rng);
     MCK(cudaMemcpy(net->idx, perm.data(), n * 4, cudaMemcpyHostToDevice));
@@ -838,26 +826,14 @@ int mw3_mlp_train(mw3_mlp* net, const float* X, const float* y, long n, int epoc
       cudaFree(dloss);
       return mfail(net, MW3_ERR_CUDA, "mw3_mlp_train: loss read-back failed");
     }
-    int updates = 0;
-    if (net->wp && (st = tc_check(net, &updates))) {   // the network stays at its last whole step
-      net->step = step0 + updates;
-      cudaFree(dloss);
-      return st;
-    }
     double sum = 0;
     for (long i = 0; i < cnt; ++i) sum += hloss[i];
     last = cnt ? sum / cnt : 0;
   }
   cudaFree(dloss);
   MCK(cudaDeviceSynchronize());
+  if (net->wp && (st = tc_check(net))) return st;
   if (final_loss) *final_loss = last;
-  return MW3_OK;
-}
-
-int mw3_mlp_set_wait_limit(mw3_mlp* net, long polls) {
-  if (!net) return MW3_ERR_BAD_ARG;
-  if (polls < 0 || polls > (1L << 22)) return mfail(net, MW3_ERR_BAD_ARG, "the wait limit must be in 0..2^22");
-  net->wait_limit = polls;
   return MW3_OK;
 }
 

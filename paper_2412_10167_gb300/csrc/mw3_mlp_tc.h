@@ -36,8 +36,7 @@ struct MlpArgs {
   long pstride;                   // number of parameters rounded up to a multiple of 4
   int nsplit, rc;                 // batch splits of the weight gradients, rows per split
   int train;
-  int* err;                       // [0] set on a wait that timed out, [1] counts the updates made
-  long wait_limit;                // polls of a bounded wait
+  int* err;                       // set on a wait that timed out
 };
 
 cudaError_t launch_mlp_chain(const MlpArgs& a, cudaStream_t st);
@@ -47,16 +46,14 @@ struct MlpShape {
   long hid0;
   int width, depth, wp;
 };
-// g[p] = sum of the partials in split order; with an update instead one AdamW step on p and the
-// BF16 copies (flat and operand form). After a wait that timed out it leaves everything as it is: the
-// partials are incomplete.
+// g[p] = sum of the partials in split order; with an update also one AdamW step on p and the
+// BF16 copies (flat and operand form)
 struct MlpUpdate {
   float *p, *g, *m, *v;
   __nv_bfloat16* ph;
   const unsigned char* wmask;
   MlpShape shape;
   unsigned char *Wf, *Wb;
-  int* err;                       // as in MlpArgs
   float lr, b1, b2, eps, wd, c1, c2;
   int update;
 };

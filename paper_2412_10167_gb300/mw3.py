@@ -132,7 +132,6 @@ _SIGS = {
     "mw3_mlp_destroy": (None, [C.c_void_p]),
     "mw3_mlp_last_error": (C.c_char_p, [C.c_void_p]),
     "mw3_mlp_num_params": (C.c_long, [C.c_void_p]),
-    "mw3_mlp_set_wait_limit": (C.c_int, [C.c_void_p, C.c_long]),
     "mw3_mlp_set_params": (C.c_int, [C.c_void_p, C.POINTER(C.c_double)]),
     "mw3_mlp_get_params": (C.c_int, [C.c_void_p, C.POINTER(C.c_double)]),
     "mw3_mlp_forward": (C.c_int, [C.c_void_p, C.POINTER(C.c_float), C.c_long,
