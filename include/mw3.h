@@ -458,6 +458,12 @@ int mw3_mlp_loss_grad(mw3_mlp* net, const float* X, const float* y, long n, doub
 int mw3_mlp_train(mw3_mlp* net, const float* X, const float* y, long n, int epochs, int batch,
                   double lr, double wd, unsigned long long seed, double* final_loss);
 
+/* Polls of each bounded mbarrier wait of the network's tensor-core kernels (widths up to 256), 0..2^22
+ * (default 2^22; 0, for the failure-detection test, makes every wait run out). A call in which a
+ * wait ran out returns MW3_ERR_TIMEOUT and leaves the network usable; mw3_mlp_train then leaves the
+ * parameters and moments of the last complete step. */
+int mw3_mlp_set_wait_limit(mw3_mlp* net, long polls);
+
 /* Allocation-free sums of squares, for callers that cannot call cudaMalloc (a fixed
  * memory arena, a region where allocating would stall other streams). The paper has
  * no counterpart: this is the per-J norm reduction of the propagation (its divergence

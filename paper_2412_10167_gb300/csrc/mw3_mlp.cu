@@ -277,7 +277,9 @@ struct mw3_mlp {
   long ld = 0;
   double* lossp = nullptr;
   long lossp_cap = 0;
-  int* tc_err = nullptr;
+  int* tc_err = nullptr;      // [0] a wait ran out, [1] updates made since the network was created
+  int tc_updates = 0;         // err[1] as the host expects it
+  long wait_limit = 1L << 22;
   int nsm = 152;
   std::string err;
 };
@@ -398,6 +400,7 @@ mw3::MlpArgs tc_args(const mw3_mlp* net, const float* X, const float* y, const i
   a.ld = net->ld;
   a.tpart = net->tpart;
   a.pstride = (net->nparam + 3) / 4 * 4;
+  a.wait_limit = net->wait_limit;
   a.err = net->tc_err;
   return a;
 }
@@ -442,14 +445,24 @@ mw3::MlpUpdate tc_update(const mw3_mlp* net) {
   u.shape = tc_shape(net);
   u.Wf = net->Wf;
   u.Wb = net->Wb;
+  u.err = net->tc_err;
   return u;
 }
 
-// After the stream is drained: did a bounded wait of the tensor-core kernels run out?
-int tc_check(mw3_mlp* net) {
-  int e = 0;
-  MCK(cudaMemcpy(&e, net->tc_err, sizeof(int), cudaMemcpyDeviceToHost));
-  return e ? mfail(net, MW3_ERR_TIMEOUT, "network kernels: an mbarrier wait timed out") : MW3_OK;
+// After the stream is drained: did a bounded wait of the tensor-core kernels run out? The word is
+// cleared for the next call. Updates queued after the wait were left out, so the parameters and
+// moments are those of the last complete step, and the step count (of the bias correction) follows.
+int tc_check(mw3_mlp* net, int steps = 0) {
+  int e[2] = {0, 0};
+  MCK(cudaMemcpy(e, net->tc_err, sizeof(e), cudaMemcpyDeviceToHost));
+  if (!e[0]) {
+    net->tc_updates += steps;
+    return MW3_OK;
+  }
+  MCK(cudaMemset(net->tc_err, 0, sizeof(int)));
+  net->step -= steps - (e[1] - net->tc_updates);
+  net->tc_updates = e[1];
+  return mfail(net, MW3_ERR_TIMEOUT, "network kernels: an mbarrier wait timed out");
 }
 
 dim3 tgrid(int M, int N, int nsplit = 1) {
@@ -553,10 +566,10 @@ int create_tc(mw3_mlp* net) {
   const size_t bytes = std::max<size_t>((size_t)(net->depth - 1) * net->wp * net->wp * 2, 16);
   MCK(cudaMalloc(&net->Wf, bytes));
   MCK(cudaMalloc(&net->Wb, bytes));
-  MCK(cudaMalloc(&net->tc_err, sizeof(int)));
+  MCK(cudaMalloc(&net->tc_err, 2 * sizeof(int)));
   MCK(cudaMemset(net->Wf, 0, bytes));
   MCK(cudaMemset(net->Wb, 0, bytes));
-  MCK(cudaMemset(net->tc_err, 0, sizeof(int)));
+  MCK(cudaMemset(net->tc_err, 0, 2 * sizeof(int)));
   return MW3_OK;
 }
 
@@ -643,6 +656,12 @@ void mw3_mlp_destroy(mw3_mlp* net) {
   cudaFree(net->lossp);
   cudaFree(net->tc_err);
   delete net;
+}
+
+int mw3_mlp_set_wait_limit(mw3_mlp* net, long polls) {
+  if (!net || polls < 0 || polls > (1L << 22)) return MW3_ERR_BAD_ARG;
+  net->wait_limit = polls;
+  return MW3_OK;
 }
 
 const char* mw3_mlp_last_error(const mw3_mlp* net) { return net ? net->err.c_str() : ""; }
@@ -762,6 +781,7 @@ int mw3_mlp_train(mw3_mlp* net, const float* X, const float* y, long n, int epoc
   std::vector<int> perm(n);
   std::iota(perm.begin(), perm.end(), 0);
   double last = 0;
+  long steps = 0;
   const float b1 = 0.9f, b2 = 0.999f;
   // per-step losses stay on the device until the end of the epoch, so the steps are queued
   // without a host round trip each
@@ -776,8 +796,12 @@ int mw3_mlp_train(mw3_mlp* net, const float* X, const float* y, long n, int epoc
       const long rows = std::min<long>(batch, n - r0);
       if (net->wp) {
         mw3::MlpArgs a = tc_args(net, net->Xall, net->yall, net->idx + r0, rows);
-        st = tc_gradient(net, a, net->lossp + cnt * tiles, nullptr);
+        if ((st = tc_gradient(net, a, net->lossp + cnt * tiles, nullptr))) {
+          cudaFree(dloss);
+          return st;
+        }
         net->step += 1;
+        ++steps;
         mw3::MlpUpdate u = tc_update(net);
         u.update = 1;
         u.lr = (float)lr;
@@ -787,9 +811,9 @@ int mw3_mlp_train(mw3_mlp* net, const float* X, const float* y, long n, int epoc
         u.wd = (float)wd;
         u.c1 = 1.f - std::pow(b1, (float)net->step);
         u.c2 = 1.f - std::pow(b2, (float)net->step);
-        if (st || mw3::launch_mlp_update(net->split, a.nsplit, a.pstride, net->nparam, u, 0) != cudaSuccess) {
+        if (mw3::launch_mlp_update(net->split, a.nsplit, a.pstride, net->nparam, u, 0) != cudaSuccess) {
           cudaFree(dloss);
-          return st ? st : mfail(net, MW3_ERR_CUDA, "mw3_mlp_train: update launch failed");
+          return mfail(net, MW3_ERR_CUDA, "mw3_mlp_train: update launch failed");
         }
         ++cnt;
         if (rows < batch) break;
@@ -832,7 +856,7 @@ int mw3_mlp_train(mw3_mlp* net, const float* X, const float* y, long n, int epoc
   }
   cudaFree(dloss);
   MCK(cudaDeviceSynchronize());
-  if (net->wp && (st = tc_check(net))) return st;
+  if (net->wp && (st = tc_check(net, (int)steps))) return st;
   if (final_loss) *final_loss = last;
   return MW3_OK;
 }

@@ -36,7 +36,8 @@ struct MlpArgs {
   long pstride;                   // number of parameters rounded up to a multiple of 4
   int nsplit, rc;                 // batch splits of the weight gradients, rows per split
   int train;
-  int* err;                       // set on a wait that timed out
+  long wait_limit;                // polls of a bounded wait
+  int* err;                       // [0] set on a wait that timed out
 };
 
 cudaError_t launch_mlp_chain(const MlpArgs& a, cudaStream_t st);
@@ -47,7 +48,8 @@ struct MlpShape {
   int width, depth, wp;
 };
 // g[p] = sum of the partials in split order; with an update also one AdamW step on p and the
-// BF16 copies (flat and operand form)
+// BF16 copies (flat and operand form). A gradient from a wait that ran out is incomplete: once
+// err[0] is set nothing is updated; err[1] counts the updates made.
 struct MlpUpdate {
   float *p, *g, *m, *v;
   __nv_bfloat16* ph;
@@ -56,6 +58,7 @@ struct MlpUpdate {
   unsigned char *Wf, *Wb;
   float lr, b1, b2, eps, wd, c1, c2;
   int update;
+  int* err;
 };
 cudaError_t launch_mlp_update(const float* part, int nsplit, long pstride, long nparam,
                               const MlpUpdate& u, cudaStream_t st);

@@ -132,6 +132,7 @@ _SIGS = {
     "mw3_mlp_destroy": (None, [C.c_void_p]),
     "mw3_mlp_last_error": (C.c_char_p, [C.c_void_p]),
     "mw3_mlp_num_params": (C.c_long, [C.c_void_p]),
+    "mw3_mlp_set_wait_limit": (C.c_int, [C.c_void_p, C.c_long]),
     "mw3_mlp_set_params": (C.c_int, [C.c_void_p, C.POINTER(C.c_double)]),
     "mw3_mlp_get_params": (C.c_int, [C.c_void_p, C.POINTER(C.c_double)]),
     "mw3_mlp_forward": (C.c_int, [C.c_void_p, C.POINTER(C.c_float), C.c_long,
@@ -546,6 +547,10 @@ class MLP:
     @property
     def num_params(self):
         return lib.mw3_mlp_num_params(self.h)
+
+    def set_wait_limit(self, polls):
+        """Polls of the tensor-core kernels' bounded waits (0: every wait runs out)."""
+        self._chk(lib.mw3_mlp_set_wait_limit(self.h, polls))
 
     def get_params(self):
         p = np.zeros(self.num_params)
