@@ -277,8 +277,8 @@ struct mw3_mlp {
   long ld = 0;
   double* lossp = nullptr;
   long lossp_cap = 0;
-  int* tc_err = nullptr;      // [0] a wait ran out, [1] updates made since the network was created
-  int tc_updates = 0;         // err[1] as the host expects it
+  int* tc_err = nullptr;      // [0] a wait ran out, [1] the last update made
+  int tc_updates = 0;         // updates made since the network was created
   long wait_limit = 1L << 22;
   int nsm = 152;
   std::string err;
@@ -335,8 +335,16 @@ int ensure_cap(mw3_mlp* net, long rows) {
   return MW3_OK;
 }
 
+// Rows that pass through the network together in training: their activations (padded to 128 or 256
+// neurons) and sums per tile stay within 8 GB. All rows of a batch at once took 321 GB for 13 million
+// rows of a network of width 32 and depth 16, four times its unpadded activations.
+long tc_rows(const mw3_mlp* net, long rows) {
+  const long most = (8L << 30) / (12L * net->depth * net->wp + 64L * (net->nin + 3)) / 128 * 128;
+  return std::min(rows, most);
+}
+
 // Buffers of the tensor-core form for batches of `rows`: inputs and outputs, with `train` also
-// the activations, their gradients and the partial weight gradients.
+// the activations, their gradients and the sums per tile of tc_rows rows.
 int ensure_tc(mw3_mlp* net, long rows, bool train) {
   if (rows > net->cap) {
     cudaFree(net->X);
@@ -349,7 +357,7 @@ int ensure_tc(mw3_mlp* net, long rows, bool train) {
     MCK(cudaMalloc(&net->out, rows * sizeof(float)));
     net->cap = rows;
   }
-  const long ld = (rows + 127) / 128 * 128;
+  const long ld = (tc_rows(net, rows) + 127) / 128 * 128;
   if (train && ld > net->ld) {
     for (float** b : {&net->Ht, &net->Dt, &net->Gt, &net->tpart}) {
       cudaFree(*b);
@@ -381,7 +389,7 @@ mw3::MlpArgs tc_args(const mw3_mlp* net, const float* X, const float* y, const i
   a.X = X;
   a.y = y;
   a.idx = idx;
-  a.n = n;
+  a.n = a.ntot = n;
   a.nin = net->nin;
   a.width = net->width;
   a.depth = net->depth;
@@ -405,15 +413,22 @@ mw3::MlpArgs tc_args(const mw3_mlp* net, const float* X, const float* y, const i
   return a;
 }
 
-// One forward and backward pass of n rows: partial gradients per batch split in net->split. The
-// splits are as many as fill the SMs with the CTAs of every layer, at least 64 rows each.
+// One forward and backward pass of n rows, tc_rows at a time: partial gradients per batch split in
+// net->split. The splits of a pass are as many as fill the SMs with the CTAs of every layer, at least
+// 64 rows each; a.nsplit is their number over all passes.
 int tc_gradient(mw3_mlp* net, mw3::MlpArgs& a, double* lossp, float* out) {
-  const long rows32 = (a.n + 31) / 32 * 32;
+  const long pass = tc_rows(net, a.n), npass = (a.n + pass - 1) / pass;
   const int per = mw3::mlp_dw_ctas(net->depth, net->wp);
   const long most = std::max(1, net->nsm / per);
-  a.rc = (int)std::max<long>(64, ((rows32 + most - 1) / most + 31) / 32 * 32);
-  a.nsplit = (int)((rows32 + a.rc - 1) / a.rc);
-  const long need = (long)a.nsplit * a.pstride;
+  auto cut = [&](mw3::MlpArgs& p, long rows) {
+    const long rows32 = (rows + 31) / 32 * 32;
+    p.rc = (int)std::max<long>(64, ((rows32 + most - 1) / most + 31) / 32 * 32);
+    p.nsplit = (int)((rows32 + p.rc - 1) / p.rc);
+  };
+  mw3::MlpArgs tail = a;
+  cut(a, pass);
+  cut(tail, a.n - (npass - 1) * pass);
+  const long need = ((npass - 1) * a.nsplit + tail.nsplit) * a.pstride;
   if (need > net->split_cap) {
     cudaFree(net->split);
     net->split = nullptr;
@@ -421,12 +436,26 @@ int tc_gradient(mw3_mlp* net, mw3::MlpArgs& a, double* lossp, float* out) {
     MCK(cudaMalloc(&net->split, need * sizeof(float)));
     net->split_cap = need;
   }
-  a.part = net->split;
-  a.lossp = lossp;
-  a.out = out;
   a.train = 1;
-  MCK(mw3::launch_mlp_chain(a, 0));
-  MCK(mw3::launch_mlp_dw(a, 0));
+  long splits = 0;
+  for (long r0 = 0; r0 < a.n; r0 += pass) {
+    mw3::MlpArgs p = a;
+    p.n = std::min(pass, a.n - r0);
+    cut(p, p.n);
+    if (a.idx) {
+      p.idx = a.idx + r0;
+    } else {
+      p.X = a.X + r0 * net->nin;
+      p.y = a.y + r0;
+    }
+    p.part = net->split + splits * a.pstride;
+    p.lossp = lossp + r0 / mw3::kMlpRows;
+    p.out = out ? out + r0 : nullptr;
+    MCK(mw3::launch_mlp_chain(p, 0));
+    MCK(mw3::launch_mlp_dw(p, 0));
+    splits += p.nsplit;
+  }
+  a.nsplit = (int)splits;
   return MW3_OK;
 }
 
@@ -803,7 +832,7 @@ int mw3_mlp_train(mw3_mlp* net, const float* X, const float* y, long n, int epoc
         net->step += 1;
         ++steps;
         mw3::MlpUpdate u = tc_update(net);
-        u.update = 1;
+        u.update = net->tc_updates + (int)steps;
         u.lr = (float)lr;
         u.b1 = b1;
         u.b2 = b2;

@@ -16,7 +16,8 @@ struct MlpArgs {
   const float* X;                 // [.][nin] inputs, row idx[r] (or r) is batch row r
   const float* y;                 // targets (training)
   const int* idx;                 // row numbers of the batch, or nullptr
-  long n;                         // batch rows
+  long n;                         // batch rows of this launch
+  long ntot;                      // rows of the whole batch (the loss is their mean)
   int nin, width, depth, wp;      // wp = mlp_tc_width(width)
   int woff[kMlpMaxLayers], boff[kMlpMaxLayers];   // flat offsets of W_l, b_l
   const float* p;                 // FP32 parameters (the biases)
@@ -49,7 +50,7 @@ struct MlpShape {
 };
 // g[p] = sum of the partials in split order; with an update also one AdamW step on p and the
 // BF16 copies (flat and operand form). A gradient from a wait that ran out is incomplete: once
-// err[0] is set nothing is updated; err[1] counts the updates made.
+// err[0] is set nothing is updated; err[1] is the number of the last update made.
 struct MlpUpdate {
   float *p, *g, *m, *v;
   __nv_bfloat16* ph;
@@ -57,7 +58,7 @@ struct MlpUpdate {
   MlpShape shape;
   unsigned char *Wf, *Wb;
   float lr, b1, b2, eps, wd, c1, c2;
-  int update;
+  int update;                     // its number, from 1 on; 0: the sum alone
   int* err;
 };
 cudaError_t launch_mlp_update(const float* part, int nsplit, long pstride, long nparam,
