@@ -446,13 +446,14 @@ bool cols_w(const T* q, T* t, long nplanes, int NR, const void* tw, const void* 
   }
 }
 
-// Half-warp form (FP32, N = 16 N1): the pair transform and its tables are in mw3_wdft.cuh.
+// Half-warp form (FP32, N = 16 N1), spectral partners by shuffles: the pair transform and its tables
+// are in mw3_wdft.cuh.
 
 // R direction, persistent: blocks of 32 rows (16 line pairs, one per half-warp of the 256
 // threads), the next block copied into the second buffer with cp.async while this one
 // transforms. Row pitch N + 8 floats: the rows of the two half-warps of a warp start 16
 // banks apart, so their exchanges do not collide.
-template <int N1, bool SHFL>
+template <int N1>
 __global__ void __launch_bounds__(256, 3) k_rows_hw(const float* __restrict__ q, float* __restrict__ t,
                                                  long nrows, const cpx<float>* __restrict__ twg,
                                                  const cpx<float>* __restrict__ phg,
@@ -497,7 +498,7 @@ __global__ void __launch_bounds__(256, 3) k_rows_hw(const float* __restrict__ q,
     __syncthreads();
     float* tile = tiles + buf * ROWS * P;
     // a pair never straddles planes (nr is even), so one flag covers both rows
-    if (live[2 * hw]) hw_pair_kinetic<N1, SHFL>(tile + 2 * hw * P, tile + (2 * hw + 1) * P, 1, lane,
+    if (live[2 * hw]) hw_pair_kinetic<N1, true>(tile + 2 * hw * P, tile + (2 * hw + 1) * P, 1, lane,
                                                 tb.tw16, tb.sig, tb.fk);
     __syncthreads();
     const int nv = (int)min((long)ROWS, nrows - row0) * (N / 4);
@@ -515,7 +516,7 @@ __global__ void __launch_bounds__(256, 3) k_rows_hw(const float* __restrict__ q,
 // Tile [N][33]: with the odd pitch, the 16 rows of an exchange fall in 16 banks, and the
 // column pairs of a warp's two half-warps, (w, w + 8) and (w + 16, w + 24), start 16 banks
 // apart. Flux cut (4-way split over r) and the R_inf column come from the tile first.
-template <int N1, bool SHFL>
+template <int N1>
 __global__ void __launch_bounds__(256) k_cols_hw(
     const float* __restrict__ q, float* __restrict__ t, int NR, const cpx<float>* __restrict__ twg,
     const cpx<float>* __restrict__ phg, const float* __restrict__ lamg, int ng,
@@ -601,7 +602,7 @@ __global__ void __launch_bounds__(256) k_cols_hw(
   {
     const int h = threadIdx.x >> 4, lane = threadIdx.x & 15;
     const int ca = (h >> 1) + 16 * (h & 1);
-    hw_pair_kinetic<N1, SHFL>(tile + ca, tile + ca + 8, LD, lane, tb.tw16, tb.sig, tb.fk);
+    hw_pair_kinetic<N1, true>(tile + ca, tile + ca + 8, LD, lane, tb.tw16, tb.sig, tb.fk);
   }
   __syncthreads();
   for (int u0 = 0; u0 < PERV; u0 += CHV) {
@@ -634,7 +635,7 @@ __global__ void __launch_bounds__(256) k_cols_hw(
   }
 }
 
-template <int N1, bool SHFL>
+template <int N1>
 bool rows_hw(const float* q, float* t, long nrows, const void* tw, const void* ph,
              const float* lam, const DevBlock* blocks, int ng, int nr, cudaStream_t st,
              cudaError_t* err) {
@@ -642,22 +643,22 @@ bool rows_hw(const float* q, float* t, long nrows, const void* tw, const void* p
   const size_t sm = ((sizeof(HwTables<N1>) + 15) / 16) * 16 + 2 * 32 * (size_t)(N + 8) * sizeof(float);
   static OncePerDevice attr;
   static IntPerDevice per;
-  *err = allow_smem(attr, k_rows_hw<N1, SHFL>, sm);
+  *err = allow_smem(attr, k_rows_hw<N1>, sm);
   if (*err != cudaSuccess) return true;
   const int per_sm = per.get(current_device(), [&] {
     int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_rows_hw<N1, SHFL>, 256, sm);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_rows_hw<N1>, 256, sm);
     return std::max(n, 1);
   });
   const long nrb = (nrows + 31) / 32;
   const unsigned grid = (unsigned)std::min<long>(nrb, (long)sm_count() * per_sm);
-  k_rows_hw<N1, SHFL><<<grid, 256, sm, st>>>(q, t, nrows, static_cast<const cpx<float>*>(tw),
+  k_rows_hw<N1><<<grid, 256, sm, st>>>(q, t, nrows, static_cast<const cpx<float>*>(tw),
                                        static_cast<const cpx<float>*>(ph), lam, blocks, ng, nr);
   *err = cudaGetLastError();
   return true;
 }
 
-template <int N1, bool SHFL>
+template <int N1>
 bool cols_hw(const float* q, float* t, long nplanes, int NR, const void* tw, const void* ph,
              const float* lam, int ng, const float* wpsi, const float* wdpsi, float* cut,
              const DevBlock* blocks, const int* ncut_J, int m_inf, float* qcol, cudaStream_t st,
@@ -665,10 +666,10 @@ bool cols_hw(const float* q, float* t, long nplanes, int NR, const void* tw, con
   constexpr int N = 16 * N1;
   const size_t sm = sizeof(HwTables<N1>) + sizeof(float) * ((size_t)N * 33 + 8 * 32);
   static OncePerDevice attr;
-  *err = allow_smem(attr, k_cols_hw<N1, SHFL>, sm);
+  *err = allow_smem(attr, k_cols_hw<N1>, sm);
   if (*err != cudaSuccess) return true;
   dim3 grid((unsigned)((NR + 31) / 32), (unsigned)nplanes);
-  k_cols_hw<N1, SHFL><<<grid, 256, sm, st>>>(q, t, NR, static_cast<const cpx<float>*>(tw),
+  k_cols_hw<N1><<<grid, 256, sm, st>>>(q, t, NR, static_cast<const cpx<float>*>(tw),
                                        static_cast<const cpx<float>*>(ph), lam, ng, wpsi, wdpsi,
                                        cut, blocks, ncut_J, m_inf, qcol);
   *err = cudaGetLastError();
@@ -685,7 +686,7 @@ bool kinetic_rows_warp(int N, const T* q, T* t, long nrows, const void* tw, cons
     if (form == 3) {
       switch (N) {
 #define HW(n1) \
-  case 16 * n1: return rows_hw<n1, true>(q, t, nrows, tw, ph, lam, blocks, ng, nr, st, err);
+  case 16 * n1: return rows_hw<n1>(q, t, nrows, tw, ph, lam, blocks, ng, nr, st, err);
         HW(8) HW(12) HW(16)
 #undef HW
         default: break;
@@ -711,7 +712,7 @@ bool kinetic_cols_warp(int N, const T* q, T* t, long nplanes, int NR, const void
       switch (N) {
 #define HW(n1)                                                                                   \
   case 16 * n1:                                                                                  \
-    return cols_hw<n1, true>(q, t, nplanes, NR, tw, ph, lam, ng, wpsi, wdpsi, cut, blocks, ncut_J, \
+    return cols_hw<n1>(q, t, nplanes, NR, tw, ph, lam, ng, wpsi, wdpsi, cut, blocks, ncut_J, \
                              m_inf, qcol, st, err);
         HW(8) HW(12) HW(16)
 #undef HW
