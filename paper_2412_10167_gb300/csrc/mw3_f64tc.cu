@@ -12,11 +12,15 @@
 //     d_s in [-128, 127] (54 bits: an element of the column's own binade is exact), each held
 //     as FP16 in tensor memory; the matrix rows likewise, once, at set-up;
 //   * level l collects the digit products with i + j = l, l = 0..7. Every partial sum is an
-//     integer below 7 K 2^14 < 2^23.5 for K <= 96, so the FP32 accumulator holds it exactly; the
-//     levels left out are below 2^-60 of (column maximum) x (row maximum). (Without level 7 the
+//     integer below 7 K 2^14 < 2^23.5 for K <= 96, so the FP32 accumulator holds it exactly. The
+//     levels left out are below 2^-59 of (column maximum) x (row maximum) per term: at most 2^-53
+//     for K = 96 terms, about 2^-59 for digits of either sign. (Without level 7 the
 //     products left out add up to several 2^-53, ten times the error of an FP64 sum.)
 //   * the eight level sums are combined in 64-bit integers and rounded to FP64 once.
-// The error is that of the 54-bit operands; FP64 units do 2 operations per
+// The error is that of the 54-bit operands: 2^-54 of the column's (row's) largest element, so that an
+// element 2^-k of it keeps 54 - k bits. An FP64 sum over the column has the same bound, its rounding
+// errors being those of the largest terms, and the measured errors agree; a column is scaled by
+// itself, so that nothing is lost between columns or blocks. FP64 units do 2 operations per
 // output instead of n_gamma / 2 (after the parity split) or n_gamma.
 //
 // Parity split of the Gauss-Legendre rule as in the mixed form: T^Omega[i][n'] =

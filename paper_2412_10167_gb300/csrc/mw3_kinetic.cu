@@ -356,11 +356,14 @@ cudaError_t launch_kinetic_rows(const real* q, real* t, long nrows, const FFTPla
                                 cudaStream_t st) {
   cudaError_t err = cudaSuccess;
   // The two-level form, except for FP64 grids with few lines: there its threads are too few to fill
-  // the FP64 pipes and the forms that spread a line over 32 or more lanes finish first (R lines of
-  // 64: 576 pairs 16.6 against 28.0 us, 1728 pairs 25.9 against 29.1; of 96: 2560 pairs 52.6 against
-  // 53.5, 7680 pairs 113 against 91; r lines of 48: 768 pairs 20.4 against 26.1; of 40: 2340 pairs
-  // 30.9 against 27.9). The pairs of one block are counted, so that a J gives the same bits alone
-  // and in a batch. FP32 is faster at every size measured.
+  // the FP64 pipes and the forms that spread a line over 32 or more lanes finish first (that form
+  // against the two-level one, pairs of the whole launch; R lines of 64: 576 pairs 16.6 against
+  // 28.0 us, 1728 pairs 25.9 against 29.1; of 96: 2560 pairs 52.6 against 53.5, 7680 pairs 113 against
+  // 91; r lines of 48: 768 pairs 20.4 against 26.1; of 40: 2340 pairs 30.9 against 27.9). The line lies
+  // where one block alone breaks even: the pairs of a block are counted, not those of the launch, so
+  // that a J gives the same bits alone and in a batch. Many small blocks together therefore keep the
+  // other form although the two-level one would be the faster (the 7680 pairs above). FP32 is faster
+  // at every size measured.
   if (warp_fft == 2 && (sizeof(real) == 4 || (long)ng * nr / 2 >= kFewLines) &&
       kinetic_rows_pairs<real>(plan.N, q, t, nrows, tw, ph, lam, blocks, ng, nr, st, &err))
     return err;
